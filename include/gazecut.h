@@ -407,8 +407,8 @@ GS_API int gs_block_descent(const int32_t *cost, const gs_params *p, int32_t b,
                             int32_t passes, int32_t *status, void *stream);
 
 /* Tile shape the TILED engine uses for these params and options: host
- * int32[4] = {sites per tile along W, rows per tile, number of tiles, shared
- * bytes}.  GS_ERR_INVAL if the requested shape does not fit. */
+ * int32[4] = {sites per tile along W, rows per tile, number of tiles, bytes of
+ * the tile's nine fields in shared memory}.  GS_ERR_INVAL if the requested shape does not fit. */
 GS_API int gs_tile_info(const gs_params *p, const gs_solve_opts *o, int32_t *out);
 
 /* Number of kernels this library has launched in this process so far. */

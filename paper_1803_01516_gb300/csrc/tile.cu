@@ -16,9 +16,9 @@
 //                   (positive excess, finite height); zero active nodes means
 //                   the preflow is maximum and the solve ends.
 //   sweep rounds    every tile with active nodes runs up to `local_iters`
-//                   push/relabel iterations in shared memory; pushes to halo
-//                   nodes go to global memory at once, and the tile writes its
-//                   own changes back as deltas, so concurrent tiles compose.
+//                   push/relabel iterations in shared memory, and writes its
+//                   changes -- its own words and what it pushed into its halo
+//                   -- back as deltas, so concurrent tiles compose.
 //
 // Correctness does not depend on the interleaving: every push moves at most
 // the excess and the residual its tile can see, and both only grow under
@@ -32,20 +32,18 @@
 namespace gs {
 
 constexpr int kTileThreads = 512;            // threads per block (256 on request: two per SM)
-constexpr int kInitOuter = 2;                 // relaxation rounds of a first relabel pass
-constexpr int kMaxTileNodes = 4096;           // own nodes per tile (8 per thread at most)
+constexpr int kInitOuter = 8;                 // relaxation rounds of a first relabel pass
+constexpr int kBlk = 4;                       // chain layers of a thread's block of own nodes
 
 struct TileGeom {
     int TW, TH;        // sites per tile along W and y
-    int PW;            // padded row length TW + 2
-    int SJ;            // shared-memory stride of one chain layer (= PW)
-    int SYs;           // shared-memory stride of one row of sites: K * PW, padded
-                       // to SYs = TW (mod 32) when R > 0
-    int PN;            // padded nodes per tile (TH + 2) * SYs
-    int TN;            // own nodes per tile TH * K * TW
-    int R;             // rows of sites one warp covers (32 / TW), 0: layers instead
-    int spread;        // R > 0: warp group g of the tile holds row group (g * spread) mod
-                       // (TN / 32), so a warp's groups lie far apart in the tile
+    int SJ;            // shared-memory stride of one field of one chain layer: TW + 2
+    int SYs;           // shared-memory stride of one row of sites: (K + 1) * 9 * SJ, padded
+                       // so that a warp's lanes fall on different banks
+    int words;         // shared words of a tile: (TH + 2) rows and kBlk layers
+    int S, nblk;       // sites of a tile, blocks of kBlk layers of a chain
+    int TN;            // own nodes per tile S * K
+    unsigned rTH, rS;  // ceil(2^32 / TH) (0 when TH = 1) and ceil(2^32 / S), for divisions
     int tiles_w, tiles_h, T;
 };
 
@@ -69,7 +67,7 @@ struct SolveArgs {
     int64_t *flow;       // label extraction output [1]
     int mode, sweeps_per_relabel, local_iters, relabel_passes, tail_iters;
     long long fixed_sweeps, max_iters;
-    int npt;             // own nodes per thread of the pair's tile shape (4 or 8)
+    int tpt;             // blocks of own nodes per thread of the pair's tile shape (1 or 2)
 };
 
 // Every read of solver state inside the persistent kernel bypasses L1: other
@@ -111,6 +109,12 @@ __device__ __forceinline__ unsigned long long atom_add_acquire(unsigned long lon
     asm volatile("atom.acquire.gpu.global.add.u64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(v) : "memory");
     return r;
 }
+__device__ __forceinline__ unsigned long long atom_add_relaxed(unsigned long long *p,
+                                                             unsigned long long v) {
+    unsigned long long r;
+    asm volatile("atom.relaxed.gpu.global.add.u64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(v) : "memory");
+    return r;
+}
 __device__ __forceinline__ unsigned long long atom_exch_release(unsigned long long *p,
                                                               unsigned long long v) {
     unsigned long long r;
@@ -119,97 +123,65 @@ __device__ __forceinline__ unsigned long long atom_exch_release(unsigned long lo
 }
 
 // ------------------------------------------------------- tile addressing ---
+//
+// A tile in shared memory: rows of sites (TH own rows and one halo row on
+// either side), in a row its K chain layers, in a layer the nine fields, in a
+// field TW + 2 sites.  The offsets from a node's cell to its 14 neighbours and
+// to the words of its arcs are then compile-time constants (tile width TWC)
+// around three addresses -- the node's cell, the one a row up and the one a
+// row down -- and go into the load instructions.  With one array per field
+// they were 28 run-time offsets, each an add and, for arcs that may not
+// exist, a select.  Between the rows lies a layer of padding whose words all
+// hold kInfH (build_tables): the layers past a chain's ends have infinite
+// heights, like the positions outside the grid, so an arc that does not exist
+// is never admissible and never gives a minimum, whatever its residual reads.
+// A thread's own nodes are blocks of kBlk consecutive layers of one site:
+// block n of a tile (n = threadIdx.x, and threadIdx.x + blockDim.x when a tile
+// has more blocks than threads) is site n mod S, layers kBlk (n / S) onwards,
+// so a warp's lanes are neighbouring sites of one row of blocks.
 
-struct TileSmem {
-    int32_t *ht, *ex, *rc, *rr, *rd, *ri0, *ri1, *ri2, *ri3;
+enum { F_EX = 0, F_HT, F_RC, F_RR, F_RD, F_I0, F_I1, F_I2, F_I3, F_N };
+
+// Strides of a tile whose width is TWC at compile time (0: at run time).
+template <int TWC>
+struct Lay {
+    int sy, sj_;
+    __device__ __forceinline__ explicit Lay(const TileGeom &t) : sy(t.SYs), sj_(t.SJ) {}
+    __device__ __forceinline__ int sj() const { return TWC ? TWC + 2 : sj_; }
+    // word offset of field f at (dj, dw) from a cell of the same row
+    __device__ __forceinline__ int at(int f, int dj = 0, int dw = 0) const {
+        return (f + F_N * dj) * sj() + dw;
+    }
+    // cell of tile position (yl, j, wl), yl in [-1, TH], wl in [-1, TW]
+    __device__ __forceinline__ int cell(int yl, int j, int wl) const {
+        return (yl + 1) * sy + (j + 1) * F_N * sj() + (wl + 1);
+    }
 };
 
-__device__ __forceinline__ TileSmem tile_smem(int32_t *base, int PN) {
-    TileSmem m;
-    m.ht = base;
-    m.ex = base + PN;
-    m.rc = base + 2 * PN;
-    m.rr = base + 3 * PN;
-    m.rd = base + 4 * PN;
-    m.ri0 = base + 5 * PN;
-    m.ri1 = base + 6 * PN;
-    m.ri2 = base + 7 * PN;
-    m.ri3 = base + 8 * PN;
-    return m;
-}
+template <int TWC>
+__device__ __forceinline__ int tile_w(const TileGeom &t) { return TWC ? TWC : t.TW; }
 
-// shared-memory index of tile position (yl, j, wl), yl in [-1, TH], wl in [-1, TW]
-__device__ __forceinline__ int pidx(const TileGeom &t, int yl, int j, int wl) {
-    return (yl + 1) * t.SYs + j * t.SJ + (wl + 1);
-}
-
-// slot -> (dy, dj, dw)
-__device__ __forceinline__ void slot_delta(int q, int &dy, int &dj, int &dw) {
-    switch (q) {
-        case 0: dy = 0; dj = 1; dw = 0; return;
-        case 1: dy = 0; dj = -1; dw = 0; return;
-        case 2: dy = 0; dj = 0; dw = 1; return;
-        case 3: dy = 0; dj = 0; dw = -1; return;
-        case 4: dy = 1; dj = 0; dw = 0; return;
-        case 5: dy = -1; dj = 0; dw = 0; return;
-        case 6: dy = 0; dj = -1; dw = -1; return;
-        case 7: dy = 0; dj = -1; dw = 1; return;
-        case 8: dy = -1; dj = -1; dw = 0; return;
-        case 9: dy = 1; dj = -1; dw = 0; return;
-        case 10: dy = 0; dj = 1; dw = -1; return;
-        case 11: dy = 0; dj = 1; dw = 1; return;
-        case 12: dy = -1; dj = 1; dw = 0; return;
-        default: dy = 1; dj = 1; dw = 0; return;
-    }
-}
-
-__device__ __forceinline__ int soff(const TileGeom &t, int q) {
-    int dy, dj, dw;
-    slot_delta(q, dy, dj, dw);
-    return dy * t.SYs + dj * t.SJ + dw;
-}
-
-// Which arcs of a node exist (grid border, chain ends, vertical inhibit off).
-__device__ __forceinline__ unsigned arc_exists(const Geom &g, int y, int j, int W) {
-    const bool up = j < g.K - 1, dn = j > 0;
-    const bool l = W > 0, r = W < g.ng - 1, u = y > 0, d = y < g.h - 1;
-    unsigned m = 0;
-    m |= up ? 1u << 0 : 0;
-    m |= dn ? 1u << 1 : 0;
-    m |= r ? 1u << 2 : 0;
-    m |= l ? 1u << 3 : 0;
-    m |= d ? 1u << 4 : 0;
-    m |= u ? 1u << 5 : 0;
-    m |= (dn && l) ? 1u << 6 : 0;
-    m |= (dn && r) ? 1u << 7 : 0;
-    m |= (dn && u) ? 1u << 8 : 0;
-    m |= (dn && d) ? 1u << 9 : 0;
-    m |= (up && l) ? 1u << 10 : 0;
-    m |= (up && r) ? 1u << 11 : 0;
-    m |= (up && u) ? 1u << 12 : 0;
-    m |= (up && d) ? 1u << 13 : 0;
-    return m;
-}
-
-// Residual of slot q of the node at shared index pi (arc known to exist).
-__device__ __forceinline__ int32_t smem_residual(const TileSmem &m, const TileGeom &t,
-                                                 const Geom &g, int pi, int q) {
-    switch (q) {
-        case 0: return m.rc[pi];
-        case 1: return kInfR;
-        case 2: return m.rr[pi];
-        case 3: return g.lam2 - m.rr[pi - 1];
-        case 4: return m.rd[pi];
-        case 5: return g.lam2 - m.rd[pi - t.SYs];
-        case 6: return m.ri0[pi];
-        case 7: return m.ri1[pi];
-        case 8: return m.ri2[pi];
-        case 9: return m.ri3[pi];
-        case 10: return g.h2h - m.ri1[pi - 1 + t.SJ];
-        case 11: return g.h2h - m.ri0[pi + 1 + t.SJ];
-        case 12: return g.h2v - m.ri3[pi - t.SYs + t.SJ];
-        default: return g.h2v - m.ri2[pi + t.SYs + t.SJ];
-    }
+// Residuals of the 14 slots of cell c (anything for an arc that does not
+// exist: its head's height is infinite).
+template <int TWC>
+__device__ __forceinline__ void load_residuals(const Lay<TWC> &l, const Geom &g,
+                                               const volatile int32_t *c,
+                                               int32_t (&r)[kSlots]) {
+    const volatile int32_t *u = c - l.sy, *d = c + l.sy;
+    r[0] = c[l.at(F_RC)];
+    r[1] = kInfR;
+    r[2] = c[l.at(F_RR)];
+    r[3] = g.lam2 - c[l.at(F_RR, 0, -1)];
+    r[4] = c[l.at(F_RD)];
+    r[5] = g.lam2 - u[l.at(F_RD)];
+    r[6] = c[l.at(F_I0)];
+    r[7] = c[l.at(F_I1)];
+    r[8] = c[l.at(F_I2)];
+    r[9] = c[l.at(F_I3)];
+    r[10] = g.h2h - c[l.at(F_I1, 1, -1)];
+    r[11] = g.h2h - c[l.at(F_I0, 1, 1)];
+    r[12] = g.h2v - u[l.at(F_I3, 1)];
+    r[13] = g.h2v - d[l.at(F_I2, 1)];
 }
 
 // Fire-and-forget adds (PTX red): no result comes back, so a push does not
@@ -218,55 +190,46 @@ __device__ __forceinline__ void red_add_smem(int32_t *p, int32_t v) {
     asm volatile("red.shared.add.s32 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(p)),
                  "r"(v));
 }
+// Shared memory by 32-bit address, under a predicate: a discharge has no
+// branches (each took longer than the access it guarded).
+__device__ __forceinline__ int32_t lds(unsigned a) {
+    int32_t r;
+    asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(r) : "r"(a));
+    return r;
+}
+__device__ __forceinline__ void sts(unsigned a, int32_t v) {
+    asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(a), "r"(v));
+}
+__device__ __forceinline__ void sts16(unsigned a, int v) {
+    asm volatile("{ .reg .b16 h; cvt.u16.u32 h, %1; st.volatile.shared.u16 [%0], h; }" ::"r"(a),
+                 "r"(v));
+}
+__device__ __forceinline__ int32_t atom_add_nz(unsigned a, int32_t v) {
+    int32_t r;
+    asm volatile("{ .reg .pred q; setp.ne.s32 q, %2, 0; mov.s32 %0, 0;"
+                 "  @q atom.shared.add.s32 %0, [%1], %2; }" : "=&r"(r) : "r"(a), "r"(v));
+    return r;
+}
+// Add w to the word at a, and v to the one at b, each if it is not 0; returns what b held
+// before (0 if it was left alone).
+__device__ __forceinline__ int32_t push_words(unsigned a, int32_t w, unsigned b, int32_t v) {
+    int32_t r;
+    asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %2, 0; setp.ne.s32 q, %4, 0; mov.s32 %0, 0;"
+                 "  @p red.shared.add.s32 [%1], %2; @q atom.shared.add.s32 %0, [%3], %4; }"
+                 : "=&r"(r) : "r"(a), "r"(w), "r"(b), "r"(v));
+    return r;
+}
+// Add v to a global word unless it is 0, and store v where p holds: no branch.
+__device__ __forceinline__ void red_add_nz(int32_t *a, int32_t v) {
+    asm volatile("{ .reg .pred p; setp.ne.s32 p, %1, 0;"
+                 "  @p red.relaxed.gpu.global.add.s32 [%0], %1; }" ::"l"(a), "r"(v));
+}
+__device__ __forceinline__ void stg_if(bool p, int32_t *a, int32_t v) {
+    asm volatile("{ .reg .pred p; setp.ne.s32 p, %2, 0; @p st.global.cg.s32 [%0], %1; }" ::"l"(a),
+                 "r"(v), "r"((int)p));
+}
 __device__ __forceinline__ void red_add_gmem(int32_t *p, int32_t v) {
     asm volatile("red.relaxed.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v));
-}
-
-// Apply a push of d along slot q to the residual words in shared memory; when
-// the word belongs to a halo node (slots whose residual is stored at the arc's
-// head), the global copy is updated at once as well.  Only the data-arc
-// residual can grow without a bound of its own (flow pushed back along the
-// infinite reverse arc); it is checked for overflow when the tile is written
-// back.  Every other word is a residual of an arc pair and stays within the
-// pair's capacity.
-__device__ __forceinline__ void smem_push_residual(const TileSmem &m, const TileGeom &t,
-                                                   const State &s, int pi, int64_t gi,
-                                                   const Geom &g, int q, int32_t d,
-                                                   bool head_is_halo) {
-    switch (q) {
-        case 0: red_add_smem(&m.rc[pi], -d); return;
-        case 1: red_add_smem(&m.rc[pi - t.SJ], d); return;   // chain never leaves the tile
-        case 2: red_add_smem(&m.rr[pi], -d); return;
-        case 3:
-            if (head_is_halo) red_add_gmem(&s.rr[gi - 1], d);
-            red_add_smem(&m.rr[pi - 1], d);
-            return;
-        case 4: red_add_smem(&m.rd[pi], -d); return;
-        case 5:
-            if (head_is_halo) red_add_gmem(&s.rd[gi - g.SY], d);
-            red_add_smem(&m.rd[pi - t.SYs], d);
-            return;
-        case 6: red_add_smem(&m.ri0[pi], -d); return;
-        case 7: red_add_smem(&m.ri1[pi], -d); return;
-        case 8: red_add_smem(&m.ri2[pi], -d); return;
-        case 9: red_add_smem(&m.ri3[pi], -d); return;
-        case 10:
-            if (head_is_halo) red_add_gmem(&s.ri1[gi - 1 + g.P], d);
-            red_add_smem(&m.ri1[pi - 1 + t.SJ], d);
-            return;
-        case 11:
-            if (head_is_halo) red_add_gmem(&s.ri0[gi + 1 + g.P], d);
-            red_add_smem(&m.ri0[pi + 1 + t.SJ], d);
-            return;
-        case 12:
-            if (head_is_halo) red_add_gmem(&s.ri3[gi - g.SY + g.P], d);
-            red_add_smem(&m.ri3[pi - t.SYs + t.SJ], d);
-            return;
-        default:
-            if (head_is_halo) red_add_gmem(&s.ri2[gi + g.SY + g.P], d);
-            red_add_smem(&m.ri2[pi + t.SYs + t.SJ], d);
-            return;
-    }
 }
 
 struct TileOrigin {
@@ -289,33 +252,38 @@ __device__ __forceinline__ TileOrigin tile_origin(const TileGeom &t, int tile) {
 // loaded afterwards by halo_rest.
 struct HaloRegs {
     int32_t h[2], r1[2], r2[2];
-    int pi[2], kind[2];
-    bool ok[2];
+    int cell[2], kind[2];      // kind -1: no cell
 };
 
 // Halo cell n of the combined index space: the left and right columns
 // (2 TH K cells), then the top and bottom rows (2 K TW cells).  kind 0..3 =
 // left, right, top, bottom.
-__device__ __forceinline__ void halo_cell(const Geom &g, const TileGeom &t, const TileOrigin &o,
-                                          int n, int &pi, int64_t &gi, bool &in, int &kind) {
+template <int TWC>
+__device__ __forceinline__ void halo_cell(const Geom &g, const TileGeom &t, const Lay<TWC> &l,
+                                          const TileOrigin &o, int n, int &cell, int64_t &gi,
+                                          bool &in, int &kind) {
+    const int TW = tile_w<TWC>(t);
     const int ncol = 2 * t.TH * g.K;
     int yl, j, wl;
     if (n < ncol) {
-        const int side = n / (t.TH * g.K), r = n - side * t.TH * g.K;
-        yl = r / g.K;
-        j = r - yl * g.K;
-        wl = side ? t.TW : -1;
-        kind = side;
+        kind = n & 1;
+        j = t.rTH ? (int)__umulhi((unsigned)(n >> 1), t.rTH) : n >> 1;
+        yl = (n >> 1) - j * t.TH;
+        wl = kind ? TW : -1;
     } else {
         n -= ncol;
-        const int side = n / (g.K * t.TW), r = n - side * g.K * t.TW;
-        j = r / t.TW;
-        wl = r - j * t.TW;
-        yl = side ? t.TH : -1;
-        kind = 2 + side;
+        j = n / TW;
+        wl = n - j * TW;
+        kind = 2;
+        yl = -1;
+        if (j >= g.K) {
+            j -= g.K;
+            kind = 3;
+            yl = t.TH;
+        }
     }
     const int W = o.W0 + wl, y = o.y0 + yl;
-    pi = pidx(t, yl, j, wl);
+    cell = l.cell(yl, j, wl);
     in = W >= 0 && W < g.ng && y >= 0 && y < g.h;
     gi = ((int64_t)y * g.K + j) * g.P + W;
 }
@@ -344,82 +312,100 @@ __device__ __forceinline__ void halo_load(const SolveArgs &a, const int32_t *hsr
     }
 }
 
-__device__ __forceinline__ void halo_store(const TileSmem &m, bool with_res, int pi, int kind,
-                                           int32_t h, int32_t r1, int32_t r2) {
-    m.ht[pi] = h;
+// Fields of a halo cell that hold the words of arcs from the tile's own nodes
+// (by kind, -1: none), the arrays they come from, and two fields it does not
+// use, where a sweep visit keeps the words as loaded.  Its excess field adds
+// up the flow a sweep visit pushes into it, from 1: a halo node always looks as
+// if it had excess before a push, so it never joins the visit's active nodes.
+__device__ __forceinline__ int halo_f1(int kind) {
+    return kind == 0 ? F_RR : kind == 1 ? F_I0 : kind == 2 ? F_RD : F_I2;
+}
+__device__ __forceinline__ int halo_f2(int kind) { return kind == 0 ? F_I1 : kind == 2 ? F_I3 : -1; }
+enum { F_KEEP1 = F_RC, F_KEEP2_COL = F_RD, F_KEEP2_ROW = F_RR };
+__device__ __forceinline__ int halo_k2(int kind) { return kind == 0 ? F_KEEP2_COL : F_KEEP2_ROW; }
+
+template <int TWC>
+__device__ __forceinline__ void halo_store(int32_t *sm, const Lay<TWC> &l, bool with_res, int cell,
+                                           int kind, int32_t h, int32_t r1, int32_t r2) {
+    int32_t *c = sm + cell;
+    c[l.at(F_HT)] = h;
     if (!with_res) return;
-    if (kind == 0) {
-        m.rr[pi] = r1;
-        m.ri1[pi] = r2;
-    } else if (kind == 1) {
-        m.ri0[pi] = r1;
-    } else if (kind == 2) {
-        m.rd[pi] = r1;
-        m.ri3[pi] = r2;
-    } else {
-        m.ri2[pi] = r1;
+    c[l.at(F_EX)] = 1;
+    c[l.at(halo_f1(kind))] = r1;
+    c[l.at(F_KEEP1)] = r1;
+    if (halo_f2(kind) >= 0) {
+        c[l.at(halo_f2(kind))] = r2;
+        c[l.at(halo_k2(kind))] = r2;
     }
 }
 
+template <int TWC>
 __device__ __forceinline__ int halo_cells(const Geom &g, const TileGeom &t) {
-    return 2 * t.TH * g.K + 2 * g.K * t.TW;
+    return 2 * g.K * (t.TH + tile_w<TWC>(t));
 }
 
-__device__ __forceinline__ void halo_issue(const SolveArgs &a, const TileOrigin &o, bool with_res,
+template <int TWC>
+__device__ __forceinline__ void halo_issue(const SolveArgs &a, const Lay<TWC> &l,
+                                           const TileOrigin &o, bool with_res,
                                            const int32_t *hsrc, HaloRegs &hr) {
-    const int total = halo_cells(a.g, a.t);
+    const int total = halo_cells<TWC>(a.g, a.t);
 #pragma unroll
     for (int u = 0; u < 2; u++) {
         const int n = threadIdx.x + u * blockDim.x;
-        hr.ok[u] = n < total;
-        hr.pi[u] = 0;
-        hr.kind[u] = 0;
+        hr.cell[u] = 0;
+        hr.kind[u] = -1;
         hr.h[u] = kInfH;
         hr.r1[u] = hr.r2[u] = 0;
-        if (!hr.ok[u]) continue;
+        if (n >= total) continue;
         int64_t gi;
         bool in;
-        halo_cell(a.g, a.t, o, n, hr.pi[u], gi, in, hr.kind[u]);
+        halo_cell<TWC>(a.g, a.t, l, o, n, hr.cell[u], gi, in, hr.kind[u]);
         halo_load(a, hsrc, with_res, gi, in, hr.kind[u], hr.h[u], hr.r1[u], hr.r2[u]);
     }
 }
 
-__device__ __forceinline__ void halo_commit(const TileSmem &m, bool with_res, const HaloRegs &hr) {
+template <int TWC>
+__device__ __forceinline__ void halo_commit(int32_t *sm, const Lay<TWC> &l, bool with_res,
+                                            const HaloRegs &hr) {
 #pragma unroll
     for (int u = 0; u < 2; u++)
-        if (hr.ok[u]) halo_store(m, with_res, hr.pi[u], hr.kind[u], hr.h[u], hr.r1[u], hr.r2[u]);
+        if (hr.kind[u] >= 0)
+            halo_store<TWC>(sm, l, with_res, hr.cell[u], hr.kind[u], hr.h[u], hr.r1[u], hr.r2[u]);
 }
 
-__device__ void halo_rest(const SolveArgs &a, const TileSmem &m, const TileOrigin &o,
+template <int TWC>
+__device__ __forceinline__ void halo_rest(const SolveArgs &a, int32_t *sm, const Lay<TWC> &l, const TileOrigin &o,
                           bool with_res, const int32_t *hsrc) {
-    const int total = halo_cells(a.g, a.t);
+    const int total = halo_cells<TWC>(a.g, a.t);
     for (int n = threadIdx.x + 2 * blockDim.x; n < total; n += blockDim.x) {
-        int pi, kind;
+        int cell, kind;
         int64_t gi;
         bool in;
-        halo_cell(a.g, a.t, o, n, pi, gi, in, kind);
+        halo_cell<TWC>(a.g, a.t, l, o, n, cell, gi, in, kind);
         int32_t h, r1, r2;
         halo_load(a, hsrc, with_res, gi, in, kind, h, r1, r2);
-        halo_store(m, with_res, pi, kind, h, r1, r2);
+        halo_store<TWC>(sm, l, with_res, cell, kind, h, r1, r2);
     }
 }
 
-// Per-block tables of the tile shape of the pair a block is working on,
-// rebuilt only when the block moves to another pair (k_batch): for every own
-// position n of a tile its shared index and coordinates, packed as
-//   p (bits 0-12) | wl (13-17) | yl (18-20) | j (21-31)
-// (shared index < 8192: a tile's 9 fields fit the 180 KB budget; wl < 32,
-// yl < 8, j < 2048), and the per-slot push table of the sweep visits.  Visits
-// then need no division to place a node.
-__shared__ uint32_t s_info[kMaxTileNodes];
+// A thread's block of own nodes: its site, first layer and number of layers
+// (0: the thread has no such block).
+struct Own {
+    int wl, yl, j0, n;
+};
 
-__device__ __forceinline__ uint32_t pack_info(int p, int wl, int yl, int j) {
-    return (uint32_t)p | ((uint32_t)wl << 13) | ((uint32_t)yl << 18) | ((uint32_t)j << 21);
+template <int TWC>
+__device__ __forceinline__ Own own_block(const Geom &g, const TileGeom &t, int u) {
+    const int id = threadIdx.x + u * blockDim.x;
+    const int blk = (int)__umulhi((unsigned)id, t.rS), site = id - blk * t.S;
+    const int TW = tile_w<TWC>(t);
+    Own w;
+    w.yl = site / TW;
+    w.wl = site - w.yl * TW;
+    w.j0 = blk * kBlk;
+    w.n = min(kBlk, max(0, g.K - w.j0));
+    return w;
 }
-__device__ __forceinline__ int info_p(uint32_t v) { return (int)(v & 0x1fffu); }
-__device__ __forceinline__ int info_wl(uint32_t v) { return (int)((v >> 13) & 31u); }
-__device__ __forceinline__ int info_yl(uint32_t v) { return (int)((v >> 18) & 7u); }
-__device__ __forceinline__ int info_j(uint32_t v) { return (int)(v >> 21); }
 
 // Search direction of a relabel pass (see SolveArgs::dir).
 __device__ __forceinline__ int eff_dir(const SolveArgs &a) {
@@ -432,66 +418,144 @@ __device__ __forceinline__ int eff_dir(const SolveArgs &a) {
 // Local relaxation to the tile's fixed point.  Own nodes' residual-arc masks
 // are in registers (mk), own heights and halo heights in shared memory.
 
-template <int NPT>
-__device__ bool relax_tile(const SolveArgs &a, const TileSmem &m, const int (&pi)[NPT],
-                           const unsigned (&mk)[NPT], int first_inner = 4,
+// One word per block of layers at the end of the tile's shared memory, that of
+// block b at b + 1 (the outer two stay 0): how often a height of the block of
+// any site changed.  Cleared before the staging barrier of a relabel visit.
+__device__ __forceinline__ uint32_t *block_words(int32_t *sm, const TileGeom &t) {
+    return (uint32_t *)sm + t.words;
+}
+__device__ __forceinline__ void clear_blocks(int32_t *sm, const TileGeom &t) {
+    uint32_t *w = block_words(sm, t);
+    for (int b = threadIdx.x; b < t.nblk + 2; b += blockDim.x) w[b] = 0;
+}
+
+// Heights of a block from those around it: a lateral minimum per node, then
+// one pass up and one pass down the block, which is exact along the chain.
+// 30 loads for four nodes instead of 14 each, and a height crosses a block of
+// the chain in one step: with one node per thread a tile of 63 layers took as
+// many dependent steps as the chain has layers (16 us a visit).  Returns
+// whether a height changed.
+template <int TWC>
+__device__ __forceinline__ bool relax_block(const Lay<TWC> &l, volatile int32_t *c, int n,
+                                            const unsigned (&mk)[kBlk]) {
+    const volatile int32_t *up = c - l.sy, *dn = c + l.sy;
+    int32_t h[kBlk], b[kBlk], L[kBlk + 2], R[kBlk + 2], U[kBlk + 2], D[kBlk + 2];
+#pragma unroll
+    for (int k = 0; k < kBlk; k++) h[k] = c[l.at(F_HT, k)];
+    const int32_t hb = c[l.at(F_HT, -1)], ha = c[l.at(F_HT, kBlk)];
+#pragma unroll
+    for (int k = 0; k < kBlk + 2; k++) {
+        L[k] = c[l.at(F_HT, k - 1, -1)];
+        R[k] = c[l.at(F_HT, k - 1, 1)];
+        U[k] = up[l.at(F_HT, k - 1)];
+        D[k] = dn[l.at(F_HT, k - 1)];
+    }
+#pragma unroll
+    for (int k = 0; k < kBlk; k++) {
+        const unsigned m = mk[k];
+        int32_t x = kInfH, y = kInfH;
+        if (m & (1u << 2)) x = min(x, R[k + 1]);
+        if (m & (1u << 3)) y = min(y, L[k + 1]);
+        if (m & (1u << 4)) x = min(x, D[k + 1]);
+        if (m & (1u << 5)) y = min(y, U[k + 1]);
+        if (m & (1u << 6)) x = min(x, L[k]);
+        if (m & (1u << 7)) y = min(y, R[k]);
+        if (m & (1u << 8)) x = min(x, U[k]);
+        if (m & (1u << 9)) y = min(y, D[k]);
+        if (m & (1u << 10)) x = min(x, L[k + 2]);
+        if (m & (1u << 11)) y = min(y, R[k + 2]);
+        if (m & (1u << 12)) x = min(x, U[k + 2]);
+        if (m & (1u << 13)) y = min(y, D[k + 2]);
+        if (k >= n) h[k] = kInfH;                 // past the chain's end
+        b[k] = min(h[k], min(x, y) + 1);
+    }
+#pragma unroll
+    for (int k = 0; k < kBlk; k++)
+        if (mk[k] & 2u) b[k] = min(b[k], (k ? b[k - 1] : hb) + 1);
+#pragma unroll
+    for (int k = kBlk - 1; k >= 0; k--)
+        if (mk[k] & 1u) b[k] = min(b[k], (k < kBlk - 1 ? b[k + 1] : ha) + 1);
+    bool ch = false;
+#pragma unroll
+    for (int k = 0; k < kBlk; k++) {
+        if (b[k] < h[k] && k < n) {
+            c[l.at(F_HT, k)] = b[k];
+            ch = true;
+        }
+    }
+    return ch;
+}
+
+template <int TPT, int TWC>
+__device__ __forceinline__ bool relax_tile(const SolveArgs &a, int32_t *sm, const int (&cell)[TPT],
+                           const int (&nl)[TPT], const unsigned (&mk)[TPT][kBlk],
                            int max_outer = 1 << 30, const unsigned *done_ctr = nullptr,
                            unsigned items = 0, bool *cut = nullptr) {
     const TileGeom &t = a.t;
-    int off[kSlots];
+    const Lay<TWC> l(t);
+    // Asynchronous (chaotic) relaxation: each warp relaxes its blocks, reading
+    // neighbours' heights as other warps update them.  Values only decrease
+    // and stay upper bounds, so any interleaving converges to the same fixed
+    // point.
+    // A block's heights depend on its own and the two adjacent blocks of
+    // layers, so a warp leaves its blocks alone unless one of these changed
+    // since it last looked (block_words): the fronts of a relaxation touch a
+    // few layers at a time.  A round ends at a barrier; one in which no height
+    // changed anywhere proves that the fixed point has been reached.  (Up to
+    // eight sweeps of a warp between barriers took 8 % longer: most warps
+    // wait for the one that goes on.)
+    const int lane = threadIdx.x & 31;
+    volatile uint32_t *chg = block_words(sm, t);
+    const bool uniform = (t.S & 31) == 0;        // a warp's blocks lie in one row of blocks
+    // lanes 16 u + i watch the i-th of the blocks around this warp's blocks u
+    // (at most 8 + 2 of them); the others watch block -1, which never changes
+    int watch = 0;
+    int blk[TPT];
 #pragma unroll
-    for (int q = 0; q < kSlots; q++) off[q] = soff(t, q);
-    // Asynchronous (chaotic) relaxation: each thread sweeps its nodes
-    // kInner times between CTA barriers, reading neighbours' heights as other
-    // warps update them.  Values only decrease and stay upper bounds, so any
-    // interleaving converges to the same fixed point; an outer round in which
-    // no height changed anywhere proves it has been reached.
-    // Neighbour heights are read with plain loads, all 14 at once (a missing
-    // arc reads the node's own height and is masked out), so they overlap:
-    // a height read stale inside a round only delays convergence, and the
-    // round that ends the loop changed nothing after fresh reads.
-    constexpr int kInner = 2;
-    int32_t *ht = m.ht;
+    for (int u = 0; u < TPT; u++) {
+        const int id0 = (threadIdx.x & ~31) + u * blockDim.x;
+        const int lo = (int)__umulhi((unsigned)id0, t.rS);
+        const int hi = min((int)__umulhi((unsigned)(id0 + 31), t.rS), t.nblk - 1);
+        blk[u] = (int)__umulhi((unsigned)(id0 + lane), t.rS);
+        const int i = lane - 16 * u;
+        if (i >= 0 && i < 16 && lo < t.nblk && i < hi - lo + 3) watch = lo + i;
+    }
+    uint32_t last = 0;
     bool any_change = false;
     // Straggler cut (with done_ctr): after a round that changed heights, stop
     // when all but 1 + min(items / 8, half the grid) of the step's items are
     // done (the last items of a step much larger than the grid are not
     // stragglers: they started late).  The caller queues the tile again, and
     // the heights so far are upper bounds of the fixed point, so a later pass
-    // resumes from them.  Thread 0 reads the done count at the start of a
-    // round and publishes its decision before the round's barrier, in a slot
-    // the next round does not overwrite.
+    // resumes from them.  Thread 0 loads the done count every other round and
+    // looks at it two rounds later (a round is shorter than the load), and
+    // publishes its decision before the round's barrier, in a slot the next
+    // round does not overwrite.
     __shared__ int s_rstop[2];
     const unsigned margin = 1 + min(items / 8, gridDim.x / 2);
+    unsigned seen = 0;
+    int stop = 0;
     for (int outer = 0;; outer++) {
         int changed = 0;
-        unsigned seen = 0;
-        if (done_ctr && threadIdx.x == 0) seen = *(volatile const unsigned *)done_ctr;
-        // a first round of fewer sweeps settles tiles whose halo change does
-        // not reach them without paying for a full round
-        const int n_inner = outer == 0 ? first_inner : kInner;
-        for (int inner = 0; inner < n_inner; inner++) {
+        if (done_ctr && threadIdx.x == 0 && (outer & 1) == 0) {
+            stop = outer >= 2 && seen + margin >= items;
+            seen = *(volatile const unsigned *)done_ctr;
+        }
+        // (the counts are read before the heights they count changes of)
+        const uint32_t now = chg[watch];
+        const bool fresh = __any_sync(0xffffffffu, now != last);
+        last = now;
+        if (fresh || outer == 0) {
 #pragma unroll
-            for (int k = 0; k < NPT; k++) {
-                if (pi[k] < 0) continue;
-                const int p = pi[k];
-                const int32_t h = ht[p];
-                if (h == 0) continue;
-                const unsigned bits = mk[k];
-                int32_t hv[kSlots];
-#pragma unroll
-                for (int q = 0; q < kSlots; q++) hv[q] = ht[p + (((bits >> q) & 1u) ? off[q] : 0)];
-                int32_t hmin = kInfH;
-#pragma unroll
-                for (int q = 0; q < kSlots; q++)
-                    if ((bits >> q) & 1u) hmin = min(hmin, hv[q]);
-                if (hmin < kInfH && hmin + 1 < h) {
-                    ht[p] = hmin + 1;
+            for (int u = 0; u < TPT; u++) {
+                const bool ch = cell[u] > 0 && relax_block<TWC>(l, sm + cell[u], nl[u], mk[u]);
+                if (__any_sync(0xffffffffu, ch)) {
                     changed = 1;
+                    if (uniform ? lane == 0 : ch) red_add_smem((int32_t *)&chg[blk[u] + 1], 1);
                 }
             }
         }
-        if (done_ctr && threadIdx.x == 0) s_rstop[outer & 1] = seen + margin >= items;
+        if (done_ctr && threadIdx.x == 0) s_rstop[outer & 1] = stop;
         if (!__syncthreads_or(changed)) break;
         any_change = true;
         if (outer + 1 >= max_outer) break;
@@ -503,116 +567,132 @@ __device__ bool relax_tile(const SolveArgs &a, const TileSmem &m, const int (&pi
     return any_change;
 }
 
+// Active count of a relabel visit and the neighbour sides it changed, zeroed
+// before the visit's staging barrier.
+__shared__ int s_count;
+__shared__ unsigned s_sides;
+
 // First relabel pass of a tile: residual-arc masks from the current state,
 // heights reset (0 on nodes with sink capacity left, else infinity), local
 // relaxation with an unknown (infinite) halo.  Returns the tile's active
 // count (positive excess and a finite height).
-template <int NPT>
-__device__ long long relabel_init_tile(const SolveArgs &a, const TileSmem &m, int tile) {
+template <int TPT, int TWC>
+__device__ __forceinline__ int relabel_init_tile(const SolveArgs &a, int32_t *sm, int tile) {
     const Geom &g = a.g;
     const TileGeom &t = a.t;
     const State &s = a.s;
+    const Lay<TWC> l(t);
     const TileOrigin o = tile_origin(t, tile);
     const int dir = eff_dir(a);
     // halo heights are not known yet in this pass: staged as infinite
     HaloRegs hr;
-    halo_issue(a, o, true, nullptr, hr);
-    int pi[NPT], pq[NPT];
-    unsigned mk[NPT];
-    int64_t gi[NPT];
-    int32_t v_rc[NPT], v_rr[NPT], v_rd[NPT], v_r0[NPT], v_r1[NPT], v_r2[NPT], v_r3[NPT], v_ex[NPT];
+    halo_issue<TWC>(a, l, o, true, nullptr, hr);
+    clear_blocks(sm, t);
+    if (threadIdx.x == 0) s_count = 0;
+    int cell[TPT], nl[TPT];      // cell > 0: a block of the grid
+    unsigned mk[TPT][kBlk];
+    int64_t gi[TPT];
+    int32_t v_rc[TPT][kBlk], v_rr[TPT][kBlk], v_rd[TPT][kBlk], v_r0[TPT][kBlk], v_r1[TPT][kBlk],
+        v_r2[TPT][kBlk], v_r3[TPT][kBlk], v_ex[TPT][kBlk];
     // own nodes: every load first ...
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        const int n = threadIdx.x + k * blockDim.x;
-        pi[k] = pq[k] = -1;
-        mk[k] = 0;
-        gi[k] = 0;
-        v_rc[k] = v_rr[k] = v_rd[k] = v_r0[k] = v_r1[k] = v_r2[k] = v_r3[k] = v_ex[k] = 0;
-        if (n >= t.TN) continue;
-        const uint32_t info = s_info[n];
-        const int wl = info_wl(info), yl = info_yl(info), j = info_j(info);
-        const int W = o.W0 + wl, y = o.y0 + yl;
-        pq[k] = info_p(info);
-        if (W >= g.ng || y >= g.h) continue;
-        const int64_t i = ((int64_t)y * g.K + j) * g.P + W;
-        pi[k] = pq[k];
-        gi[k] = i;
-        v_rc[k] = ld(&s.rc[i]);
-        v_rr[k] = ld(&s.rr[i]);
-        v_rd[k] = ld(&s.rd[i]);
-        v_r0[k] = ld(&s.ri0[i]);
-        v_r1[k] = ld(&s.ri1[i]);
-        v_r2[k] = ld(&s.ri2[i]);
-        v_r3[k] = ld(&s.ri3[i]);
-        v_ex[k] = ld(&s.ex[i]);
+    for (int u = 0; u < TPT; u++) {
+        const Own w = own_block<TWC>(g, t, u);
+        const int W = o.W0 + w.wl, y = o.y0 + w.yl;
+        nl[u] = w.n;
+        cell[u] = w.n ? l.cell(w.yl, w.j0, w.wl) : 0;
+        if (W >= g.ng || y >= g.h) cell[u] = -cell[u];
+        gi[u] = ((int64_t)y * g.K + w.j0) * g.P + W;
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) {
+            mk[u][k] = 0;
+            v_rc[u][k] = v_rr[u][k] = v_rd[u][k] = v_r0[u][k] = v_r1[u][k] = v_r2[u][k] =
+                v_r3[u][k] = v_ex[u][k] = 0;
+            if (cell[u] <= 0 || k >= nl[u]) continue;
+            const int64_t i = gi[u] + (int64_t)k * g.P;
+            v_rc[u][k] = ld(&s.rc[i]);
+            v_rr[u][k] = ld(&s.rr[i]);
+            v_rd[u][k] = ld(&s.rd[i]);
+            v_r0[u][k] = ld(&s.ri0[i]);
+            v_r1[u][k] = ld(&s.ri1[i]);
+            v_r2[u][k] = ld(&s.ri2[i]);
+            v_r3[u][k] = ld(&s.ri3[i]);
+            v_ex[u][k] = ld(&s.ex[i]);
+        }
     }
     // ... then the shared-memory stores
-    halo_commit(m, true, hr);
+    halo_commit<TWC>(sm, l, true, hr);
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        if (pq[k] < 0) continue;
-        const int p = pq[k];
-        if (pi[k] < 0) {
-            m.ht[p] = kInfH;
-            continue;
-        }
-        m.rc[p] = v_rc[k];
-        m.rr[p] = v_rr[k];
-        m.rd[p] = v_rd[k];
-        m.ri0[p] = v_r0[k];
-        m.ri1[p] = v_r1[k];
-        m.ri2[p] = v_r2[k];
-        m.ri3[p] = v_r3[k];
-        const int32_t e = v_ex[k];
-        if (dir == 0) {
-            m.ht[p] = e < 0 ? 0 : kInfH;
-            mk[k] = e > 0 ? 0x8000u : 0u;
-        } else {
-            m.ht[p] = e > 0 ? 0 : kInfH;
-        }
-    }
-    halo_rest(a, m, o, true, nullptr);
-    __syncthreads();
+    for (int u = 0; u < TPT; u++) {
+        int32_t *c = sm + abs(cell[u]);
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        if (pi[k] < 0) continue;
-        const uint32_t info = s_info[threadIdx.x + k * blockDim.x];
-        const unsigned ex = arc_exists(g, o.y0 + info_yl(info), info_j(info), o.W0 + info_wl(info));
-#pragma unroll
-        for (int q = 0; q < kSlots; q++) {
-            if (!((ex >> q) & 1u)) continue;
-            bool res;
-            if (dir == 0) {
-                res = smem_residual(m, t, g, pi[k], q) > 0;          // arc u -> head
-            } else if (q == 0) {
-                res = true;                                           // head j+1 -> u: infinite
-            } else if (q == 1) {
-                res = m.rc[pi[k] - t.SJ] > 0;                         // head j-1 -> u: data arc
-            } else {
-                const int32_t cap = q < 6 ? g.lam2 : (q == 8 || q == 9 || q == 12 || q == 13) ? g.h2v
-                                                                                             : g.h2h;
-                res = cap - smem_residual(m, t, g, pi[k], q) > 0;     // head -> u: pair reverse
+        for (int k = 0; k < kBlk; k++) {
+            if (cell[u] == 0 || k >= nl[u]) continue;
+            if (cell[u] < 0) {
+                c[l.at(F_HT, k)] = kInfH;
+                continue;
             }
-            if (res) mk[k] |= 1u << q;
+            c[l.at(F_RC, k)] = v_rc[u][k];
+            c[l.at(F_RR, k)] = v_rr[u][k];
+            c[l.at(F_RD, k)] = v_rd[u][k];
+            c[l.at(F_I0, k)] = v_r0[u][k];
+            c[l.at(F_I1, k)] = v_r1[u][k];
+            c[l.at(F_I2, k)] = v_r2[u][k];
+            c[l.at(F_I3, k)] = v_r3[u][k];
+            const int32_t e = v_ex[u][k];
+            c[l.at(F_HT, k)] = (dir == 0 ? e < 0 : e > 0) ? 0 : kInfH;
         }
-        __stcg(&a.amask[gi[k]], (uint16_t)mk[k]);
     }
+    halo_rest<TWC>(a, sm, l, o, true, nullptr);
     __syncthreads();
+#pragma unroll
+    for (int u = 0; u < TPT; u++) {
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) {
+            if (cell[u] <= 0 || k >= nl[u]) continue;
+            const int32_t *c = sm + cell[u] + l.at(0, k);
+            int32_t r[kSlots];
+            load_residuals<TWC>(l, g, c, r);
+            unsigned m = 0;
+            if (dir == 0) {
+                // arc u -> head
+#pragma unroll
+                for (int q = 0; q < kSlots; q++) m |= r[q] > 0 ? 1u << q : 0u;
+            } else {
+                // arc head -> u: the reverse of the data arc up is infinite, that
+                // of the one down is the data arc of layer j - 1, else the
+                // pair's rest
+                m = 1u | (c[l.at(F_RC, -1)] > 0 ? 2u : 0u);
+#pragma unroll
+                for (int q = 2; q < kSlots; q++) {
+                    const int32_t cap = q < 6 ? g.lam2 : q == 8 || q == 9 || q >= 12 ? g.h2v : g.h2h;
+                    m |= cap - r[q] > 0 ? 1u << q : 0u;
+                }
+            }
+            mk[u][k] = m | (dir == 0 && v_ex[u][k] > 0 ? 0x8000u : 0u);
+            __stcg(&a.amask[gi[u] + (int64_t)k * g.P], (uint16_t)mk[u][k]);
+        }
+    }
+    // (no barrier: the masks read words that only the staging wrote)
     // the first pass's relaxation is capped: the pass after it visits every
     // tile again, with the halo known, and relaxes each to its fixed point
-    relax_tile<NPT>(a, m, pi, mk, 4, kInitOuter);
+    relax_tile<TPT, TWC>(a, sm, cell, nl, mk, kInitOuter);
     int act = 0;
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        if (pi[k] < 0) continue;
-        const int32_t h = m.ht[pi[k]];
-        __stcg(&a.hgt[gi[k]], h);
-        act += (mk[k] & 0x8000u) && h < kInfH;
+    for (int u = 0; u < TPT; u++) {
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) {
+            if (cell[u] <= 0 || k >= nl[u]) continue;
+            const int32_t h = sm[cell[u] + l.at(F_HT, k)];
+            __stcg(&a.hgt[gi[u] + (int64_t)k * g.P], h);
+            act += (mk[u][k] & 0x8000u) && h < kInfH;
+        }
     }
-    const long long tot = block_sum(act);
-    if (threadIdx.x == 0) __stcg(&a.tile_cnt[tile], (int32_t)tot);
-    return tot;
+    act = __reduce_add_sync(0xffffffffu, act);
+    if ((threadIdx.x & 31) == 0 && act) atomicAdd(&s_count, act);
+    __syncthreads();
+    if (threadIdx.x == 0) __stcg(&a.tile_cnt[tile], s_count);
+    return s_count;
 }
 
 // Queue a tile for the next step, once: the caller that turns its flag from 0
@@ -632,398 +712,447 @@ __device__ __forceinline__ int side_tile(const TileGeom &t, const TileOrigin &o,
 
 // Later relabel passes: masks from the first pass, heights from global
 // memory (own and halo); relax, write back what changed, mark the neighbour
-// tiles whose halo changed, and return the change of the tile's active count.
-template <int NPT>
-__device__ long long relabel_pass_tile(const SolveArgs &a, const TileSmem &m, int tile,
-                                       int &changed, int32_t *dirty_next, int32_t *list_next,
-                                       int32_t *count_next, const unsigned *done_ctr,
-                                       unsigned items) {
+// tiles whose halo changed, and return the change of the tile's active count
+// (the marks are warp 0's and come after the visit's last block barrier).
+template <int TPT, int TWC>
+__device__ __forceinline__ int relabel_pass_tile(const SolveArgs &a, int32_t *sm, int tile, int &changed,
+                                 int32_t *dirty_next, int32_t *list_next, int32_t *count_next,
+                                 const unsigned *done_ctr, unsigned items) {
     const Geom &g = a.g;
     const TileGeom &t = a.t;
+    const Lay<TWC> l(t);
     const TileOrigin o = tile_origin(t, tile);
-    const long long before = ld(&a.tile_cnt[tile]);   // issued now, used at the end
+    const int before = ld(&a.tile_cnt[tile]);    // issued now, used at the end
     HaloRegs hr;
-    halo_issue(a, o, false, a.hgt, hr);
-    int pi[NPT], pq[NPT];
-    unsigned mk[NPT];
-    int64_t gi[NPT];
-    int32_t h0[NPT];
+    halo_issue<TWC>(a, l, o, false, a.hgt, hr);
+    clear_blocks(sm, t);
+    if (threadIdx.x == 0) {
+        s_count = 0;
+        s_sides = 0;
+    }
+    int cell[TPT], nl[TPT];      // cell > 0: a block of the grid
+    unsigned mk[TPT][kBlk];
+    int64_t gi[TPT];
+    int32_t h0[TPT][kBlk];
     // own nodes: every load first, then the shared-memory stores
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        const int n = threadIdx.x + k * blockDim.x;
-        pi[k] = pq[k] = -1;
-        mk[k] = 0;
-        gi[k] = 0;
-        h0[k] = kInfH;
-        if (n >= t.TN) continue;
-        const uint32_t info = s_info[n];
-        const int wl = info_wl(info), yl = info_yl(info), j = info_j(info);
-        const int W = o.W0 + wl, y = o.y0 + yl;
-        pq[k] = info_p(info);
-        if (W >= g.ng || y >= g.h) continue;
-        const int64_t i = ((int64_t)y * g.K + j) * g.P + W;
-        pi[k] = pq[k];
-        gi[k] = i;
-        mk[k] = ld(&a.amask[i]);
-        h0[k] = ld(&a.hgt[i]);
-    }
-    halo_commit(m, false, hr);
+    for (int u = 0; u < TPT; u++) {
+        const Own w = own_block<TWC>(g, t, u);
+        const int W = o.W0 + w.wl, y = o.y0 + w.yl;
+        nl[u] = w.n;
+        cell[u] = w.n ? l.cell(w.yl, w.j0, w.wl) : 0;
+        if (W >= g.ng || y >= g.h) cell[u] = -cell[u];
+        gi[u] = ((int64_t)y * g.K + w.j0) * g.P + W;
 #pragma unroll
-    for (int k = 0; k < NPT; k++)
-        if (pq[k] >= 0) m.ht[pq[k]] = h0[k];
-    halo_rest(a, m, o, false, a.hgt);
-    __shared__ int s_sides;
-    if (threadIdx.x == 0) s_sides = 0;
+        for (int k = 0; k < kBlk; k++) {
+            mk[u][k] = 0;
+            h0[u][k] = kInfH;
+            if (cell[u] <= 0 || k >= nl[u]) continue;
+            const int64_t i = gi[u] + (int64_t)k * g.P;
+            mk[u][k] = ld(&a.amask[i]);
+            h0[u][k] = ld(&a.hgt[i]);
+        }
+    }
+    halo_commit<TWC>(sm, l, false, hr);
+#pragma unroll
+    for (int u = 0; u < TPT; u++)
+#pragma unroll
+        for (int k = 0; k < kBlk; k++)
+            if (cell[u] && k < nl[u]) sm[abs(cell[u]) + l.at(F_HT, k)] = h0[u][k];
+    halo_rest<TWC>(a, sm, l, o, false, a.hgt);
     __syncthreads();
-    // one sweep first: most tiles a halo change marks need no more
     bool cut = false;
-    const bool ch = relax_tile<NPT>(a, m, pi, mk, 1, 1 << 30, done_ctr, items, &cut);
+    const bool ch = relax_tile<TPT, TWC>(a, sm, cell, nl, mk, 1 << 30, done_ctr, items, &cut);
     int act = 0;
     unsigned sides = 0;
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        if (pi[k] < 0) continue;
-        const int32_t h = m.ht[pi[k]];
-        if (h != h0[k]) {
-            __stcg(&a.hgt[gi[k]], h);
-            const uint32_t info = s_info[threadIdx.x + k * blockDim.x];
-            const int wl = info_wl(info), yl = info_yl(info);
-            sides |= (wl == 0 ? 1u : 0u) | (wl == t.TW - 1 ? 2u : 0u) | (yl == 0 ? 4u : 0u) |
-                     (yl == t.TH - 1 ? 8u : 0u);
+    for (int u = 0; u < TPT; u++) {
+        bool moved = false;
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) {
+            if (cell[u] <= 0 || k >= nl[u]) continue;
+            const int32_t h = sm[cell[u] + l.at(F_HT, k)];
+            if (h != h0[u][k]) {
+                __stcg(&a.hgt[gi[u] + (int64_t)k * g.P], h);
+                moved = true;
+            }
+            act += (mk[u][k] & 0x8000u) && h < kInfH;
         }
-        act += (mk[k] & 0x8000u) && h < kInfH;
+        if (moved) {
+            const Own w = own_block<TWC>(g, t, u);
+            sides |= (w.wl == 0 ? 1u : 0u) | (w.wl == tile_w<TWC>(t) - 1 ? 2u : 0u) |
+                     (w.yl == 0 ? 4u : 0u) | (w.yl == t.TH - 1 ? 8u : 0u);
+        }
     }
-    if (sides) atomicOr(&s_sides, (int)sides);
-    const long long tot = block_sum(act);   // also orders s_sides
-    if (threadIdx.x < 4 && ((unsigned)s_sides >> threadIdx.x & 1u)) {
+    act = __reduce_add_sync(0xffffffffu, act);
+    sides = __reduce_or_sync(0xffffffffu, sides);
+    if ((threadIdx.x & 31) == 0) {
+        if (act) atomicAdd(&s_count, act);
+        if (sides) atomicOr(&s_sides, sides);
+    }
+    __syncthreads();
+    if (threadIdx.x < 4 && (s_sides >> threadIdx.x & 1u)) {
         const int nb = side_tile(t, o, tile, threadIdx.x);
         if (nb >= 0) enqueue(dirty_next, list_next, count_next, nb);
     }
     // a relaxation cut short goes on in the next pass
     if (cut && threadIdx.x == 4) enqueue(dirty_next, list_next, count_next, tile);
     if (ch) changed = 1;
-    __syncthreads();
-    if (threadIdx.x == 0) __stcg(&a.tile_cnt[tile], (int32_t)tot);
-    return tot - before;
+    if (threadIdx.x == 0) __stcg(&a.tile_cnt[tile], s_count);
+    return s_count - before;
 }
 
 // ------------------------------------------------------------ sweep visit ---
 
-// Per-slot push table of a tile shape, in shared memory: where a push along
-// slot q changes the residual word (shared offset from the node, its kind and
-// the pair capacity), where the head's excess lives (shared offset, global
-// offset), and where the word lives in global memory when the head is a halo
-// node.  A discharge then loops over a node's admissible slots only -- one or
-// two on average -- instead of running the code of all 14.
-//   .x  sword  shared offset of the residual word from the node (field * PN + off)
-//   .y  sex    shared offset of the head's excess
-//   .z  kind   0: word stored at the node (r = word, a push subtracts)
-//              1: word stored at the head (r = cap - word, a push adds)
-//              2: the infinite reverse data arc (a push adds to the head's rc)
-//   .w  cap    pair capacity of kind 1
-//   [1] .x dw, .y dy (head position in the tile), .z gfield (global array of
-//       the word: 0 rc .. 6 ri3), .w grel (global offset of the word)
-//   [2] .x gex (global offset of the head)
-struct SlotTab {
-    int4 a, b, c;
-};
+// One arc slot of a tile shape; in a sweep visit a lane holds four.  Offsets
+// count from the node's cell, in bytes.
+//   .x  shared offset of the residual word
+//   .y  shared offset of the head's cell
+//   .z, .w  residual = z + w * word: 0, 1 when the word is stored at the node (a push
+//       subtracts); the pair's capacity, -1 when it is stored at the head (a push adds);
+//       infinite, 0 for the reverse data arc (a push adds to the head's word)
+// Entries 14 and 15 are no arcs: the node itself, never residual.
+__shared__ int4 s_slot[16];
 
-__device__ __forceinline__ SlotTab make_slot(const Geom &g, const TileGeom &t, int q) {
-    int dy, dj, dw;
-    slot_delta(q, dy, dj, dw);
-    const int off = dy * t.SYs + dj * t.SJ + dw;
-    // tile field order in shared memory: ht 0, ex 1, rc 2, rr 3, rd 4, ri0..ri3 5..8;
-    // in global memory: rc 0, rr 1, rd 2, ri0..ri3 3..6, ex 7, ht 8
-    int sfield, roff = 0, kind = 0, cap = 0, gfield = -1, grel = 0;
-    switch (q) {
-        case 0: sfield = 2; break;
-        case 1: sfield = 2; roff = -t.SJ; kind = 2; break;
-        case 2: sfield = 3; break;
-        case 3: sfield = 3; roff = -1; kind = 1; cap = g.lam2; gfield = 1; grel = -1; break;
-        case 4: sfield = 4; break;
-        case 5: sfield = 4; roff = -t.SYs; kind = 1; cap = g.lam2; gfield = 2; grel = -(int)g.SY; break;
-        case 6: sfield = 5; break;
-        case 7: sfield = 6; break;
-        case 8: sfield = 7; break;
-        case 9: sfield = 8; break;
-        case 10: sfield = 6; roff = -1 + t.SJ; kind = 1; cap = g.h2h; gfield = 4; grel = -1 + g.P; break;
-        case 11: sfield = 5; roff = 1 + t.SJ; kind = 1; cap = g.h2h; gfield = 3; grel = 1 + g.P; break;
-        case 12:
-            sfield = 8; roff = -t.SYs + t.SJ; kind = 1; cap = g.h2v; gfield = 6;
-            grel = -(int)g.SY + g.P;
-            break;
-        default:
-            sfield = 7; roff = t.SYs + t.SJ; kind = 1; cap = g.h2v; gfield = 5;
-            grel = (int)g.SY + g.P;
-            break;
-    }
-    SlotTab e;
-    e.a = make_int4(sfield * t.PN + roff, t.PN + off, kind, cap);
-    e.b = make_int4(dw, dy, gfield, grel);
-    e.c = make_int4((int)(dy * g.SY + (int64_t)dj * g.P + dw), 0, 0, 0);
-    return e;
+__device__ __forceinline__ int4 make_slot(const Geom &g, const TileGeom &t, int q) {
+    // head (dy, dj, dw) and field of the word
+    static constexpr int8_t tab[kSlots][4] = {
+        {0, 1, 0, F_RC},  {0, -1, 0, F_RC},  {0, 0, 1, F_RR},  {0, 0, -1, F_RR}, {1, 0, 0, F_RD},
+        {-1, 0, 0, F_RD}, {0, -1, -1, F_I0}, {0, -1, 1, F_I1}, {-1, -1, 0, F_I2}, {1, -1, 0, F_I3},
+        {0, 1, -1, F_I1}, {0, 1, 1, F_I0},   {-1, 1, 0, F_I3}, {1, 1, 0, F_I2}};
+    if (q >= kSlots) return make_int4(0, 0, 0, 0);
+    const int off = tab[q][0] * t.SYs + tab[q][1] * F_N * t.SJ + tab[q][2];
+    const bool at_head = q == 3 || q == 5 || q >= 10;
+    const int cap = q < 6 ? g.lam2 : q < 12 ? g.h2h : g.h2v;
+    return make_int4(4 * (tab[q][3] * t.SJ + (at_head || q == 1 ? off : 0)), 4 * off,
+                     q == 1 ? kInfR : at_head ? cap : 0, q == 1 ? 0 : at_head ? -1 : 1);
 }
 
-__shared__ SlotTab s_slot[kSlots];
-
-// Fill the block's tables (s_info, s_slot) for the tile shape of pair a.
-__device__ void build_tables(const SolveArgs &a) {
+// Fill the block's tables for the tile shape of pair a: s_slot, and the
+// padding between the rows of a tile.
+__device__ void build_tables(const SolveArgs &a, int32_t *sm) {
     const Geom &g = a.g;
     const TileGeom &t = a.t;
-    for (int n = threadIdx.x; n < t.TN; n += blockDim.x) {
-        int wl, yl, j;
-        if (t.R) {
-            // lanes: TW sites x R rows of one layer; the warp group g = n / 32
-            // is placed at group (g * spread) mod M, M = TN / 32, numbered
-            // layer first, then row group
-            wl = n % t.TW;
-            const int u = (n / t.TW) % t.R;
-            const int M = t.TN / 32;
-            const int gp = (int)(((long long)(n / 32) * t.spread) % M);
-            j = gp % g.K;
-            yl = (gp / g.K) * t.R + u;
-        } else {
-            wl = n % t.TW;
-            const int r = n / t.TW;
-            j = r % g.K;
-            yl = r / g.K;
-        }
-        s_info[n] = pack_info(pidx(t, yl, j, wl), wl, yl, j);
+    if (threadIdx.x < 16) s_slot[threadIdx.x] = make_slot(g, t, threadIdx.x);
+    const int layer = F_N * t.SJ, pad = t.SYs - (g.K + 1) * layer;
+    for (int r = 0; r <= t.TH + 2; r++) {
+        const int to = min(t.words, r * t.SYs + layer);
+        for (int w = max(0, r * t.SYs - pad) + threadIdx.x; w < to; w += blockDim.x) sm[w] = kInfH;
     }
-    if (threadIdx.x < kSlots) s_slot[threadIdx.x] = make_slot(g, t, threadIdx.x);
 }
 
+// Lists of a sweep visit's active nodes (positive excess, finite height), as
+// cells, for the iteration running and the next: two halves of TN entries
+// behind the block words, and one entry more that takes what goes nowhere.
+// Their lengths, by iteration mod kLens (warp 0 may run half as many ahead).
+constexpr int kLens = 64;
+__shared__ int s_nodes[kLens];
 
+// Discharge the eight nodes of a list (shared address `list`, n entries) from
+// entry `first` on, four lanes to a node: lane q of the four holds arc slots
+// 4 q .. 4 q + 3 (st), the last one also the node's own words.  A lane loads
+// its arcs' residuals and its heads' heights, a saturating scan over the four
+// lanes deals the excess out to the admissible slots in slot order (chain arcs
+// first; another order took 20 % more visits), and each lane pushes its
+// share; a minimum over the same lanes gives the relabel.  Flow into the halo
+// gathers in the halo cells' excess and words.
+// A node joins the next list when a push takes its excess above zero, or when
+// it has excess left after its own discharge: once in either case.
+// A warp is bound by the chain of dependent instructions here, and an
+// iteration has 17 to 45 active nodes on average: one lane per node ran the
+// code of 14 slots for lanes most of which were idle, and sixteen or eight
+// lanes per node took as long for two or four nodes as four lanes do for eight.
+template <int TWC>
+__device__ __forceinline__ void discharge(const Lay<TWC> &l, unsigned base, unsigned list,
+                                          int first, int n, const int4 (&st)[4], unsigned next,
+                                          unsigned next_n, unsigned nowhere) {
+    const int lane = threadIdx.x & 31, q = lane & 3;
+    const int i = first + (lane >> 2);
+    unsigned c;
+    asm volatile("{ .reg .u16 h; ld.volatile.shared.u16 h, [%1]; cvt.u32.u16 %0, h; }"
+                 : "=r"(c) : "r"(list + 2 * min(i, n - 1)));
+    c = base + 4 * c;
+    int32_t e = lds(c + 4 * l.at(F_EX));
+    const int32_t hu = lds(c + 4 * l.at(F_HT));
+    int32_t r[4], hv[4], x[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        r[j] = lds(c + st[j].x);
+        hv[j] = lds(c + st[j].y + 4 * l.at(F_HT));
+    }
+    if (i >= n) e = 0;
+    int32_t hm = kInfH;
+    unsigned sum = 0;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        r[j] = (int32_t)((unsigned)st[j].z + (unsigned)st[j].w * (unsigned)r[j]);
+        // (a head that does not exist has an infinite height)
+        x[j] = r[j] > 0 && hv[j] < hu ? min(r[j], e) : 0;
+        hm = min(hm, r[j] > 0 && hv[j] >= hu ? hv[j] : kInfH);
+        sum = min(sum + (unsigned)x[j], (unsigned)e);
+    }
+#pragma unroll
+    for (int s = 1; s < 4; s <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, sum, s, 4);
+        hm = min(hm, __shfl_xor_sync(0xffffffffu, hm, s));
+        if (q >= s) sum = min(sum + y, (unsigned)e);
+    }
+    const unsigned y = __shfl_up_sync(0xffffffffu, sum, 1, 4);
+    const bool own = q == 3;
+    const int32_t tot = (int32_t)sum;            // lane 3: all the flow pushed
+    int32_t left = e - (q ? (int32_t)y : 0), old[4];
+    unsigned ea[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        x[j] = min(x[j], left);
+        left -= x[j];
+        ea[j] = c + st[j].y + 4 * l.at(F_EX);
+        old[j] = push_words(c + st[j].x, st[j].w > 0 ? -x[j] : x[j], ea[j],
+                            j == 2 && own ? -tot : x[j]);
+    }
+    // lane 3: every admissible slot is saturated: relabel over the others
+    const bool stuck = own && tot < e;
+    const int32_t h = !stuck ? hu : hm >= kInfH - 1 ? kInfH : hm + 1;
+    sts(stuck ? c + 4 * l.at(F_HT) : nowhere, h);
+    bool join[4];
+    int joins = 0;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        join[j] = x[j] > 0 && old[j] <= 0 && old[j] + x[j] > 0;
+        if (j == 2 && own) join[j] = (tot ? old[j] - tot : e) > 0 && h < kInfH;
+        joins += join[j];
+    }
+    unsigned at = next + 2 * (unsigned)atom_add_nz(next_n, joins);
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        sts16(join[j] ? at : nowhere, (int)((ea[j] - base) >> 2));
+        if (join[j]) at += 2;
+    }
+}
 
-// Up to local_iters push/relabel iterations of one tile in shared memory.
-template <int NPT, int BT>
-__device__ void sweep_tile(const SolveArgs &a, const TileSmem &m, int tile, int round, int iters,
+// Up to `iters` push/relabel iterations of one tile in shared memory.  (The
+// queueing at the end is warp 0's and comes after the visit's last barrier.)
+template <int TPT, int TWC>
+__device__ __forceinline__ void sweep_tile(const SolveArgs &a, int32_t *sm, int tile, int round, int iters,
                            int &overflow, int32_t *list_next, int32_t *count_next,
-                           const unsigned *done_ctr, unsigned items,
-                           uint32_t (*s_wlist)[8 * 32]) {
+                           const unsigned *done_ctr, unsigned items) {
     const Geom &g = a.g;
     const TileGeom &t = a.t;
     const State &s = a.s;
+    const Lay<TWC> l(t);
     const TileOrigin o = tile_origin(t, tile);
     int32_t *act_next = a.tile_act + ((round + 1) & 1) * t.T;
-    const int64_t tile_g0 = (int64_t)o.y0 * g.SY + o.W0;
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, W = blockDim.x >> 5;
     __shared__ unsigned s_touch;
-    __shared__ int s_stop;
-    if (threadIdx.x == 0) {
-        s_touch = 0;   // read only after the staging barrier below
-        s_stop = 0;
-    }
+    __shared__ int s_stop[2];        // in turn: written before an iteration's barrier
+    __shared__ int s_it;
+    if (threadIdx.x == 0) s_touch = 0;   // read only after the staging barrier below
+    if (threadIdx.x < kLens) s_nodes[threadIdx.x] = 0;
     HaloRegs hr;
-    halo_issue(a, o, true, s.ht, hr);
-    // own node k of this thread: its packed position (s_info) and whether it
-    // lies inside the grid (bit k of vmask); positions past the tile's nodes
-    // are not in vmask either
-    uint32_t inf[NPT];
-    unsigned vmask = 0, tmask = 0;
-    int32_t o_ex[NPT], o_rc[NPT], o_rr[NPT], o_rd[NPT], o_r0[NPT], o_r1[NPT], o_r2[NPT],
-        o_r3[NPT], o_ht[NPT];
+    halo_issue<TWC>(a, l, o, true, s.ht, hr);
+    int cell[TPT], nl[TPT];      // cell > 0: a block of the grid
+    int64_t gi[TPT];
+    int32_t o_ex[TPT][kBlk], o_rc[TPT][kBlk], o_rr[TPT][kBlk], o_rd[TPT][kBlk], o_r0[TPT][kBlk],
+        o_r1[TPT][kBlk], o_r2[TPT][kBlk], o_r3[TPT][kBlk], o_ht[TPT][kBlk];
     // own nodes: every load first (the originals stay in registers for the
     // write-back as deltas) ...
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        const int n = threadIdx.x + k * blockDim.x;
-        inf[k] = 0;
-        o_ex[k] = o_rc[k] = o_rr[k] = o_rd[k] = o_r0[k] = o_r1[k] = o_r2[k] = o_r3[k] = 0;
-        o_ht[k] = kInfH;
-        if (n >= t.TN) continue;
-        const uint32_t info = s_info[n];
-        inf[k] = info;
-        tmask |= 1u << k;
-        const int W = o.W0 + info_wl(info), y = o.y0 + info_yl(info);
-        if (W >= g.ng || y >= g.h) continue;
-        vmask |= 1u << k;
-        const int64_t i = tile_g0 + (int64_t)info_yl(info) * g.SY +
-                          (int64_t)info_j(info) * g.P + info_wl(info);
-        o_ex[k] = ld(&s.ex[i]);
-        o_ht[k] = ld(&s.ht[i]);
-        o_rc[k] = ld(&s.rc[i]);
-        o_rr[k] = ld(&s.rr[i]);
-        o_rd[k] = ld(&s.rd[i]);
-        o_r0[k] = ld(&s.ri0[i]);
-        o_r1[k] = ld(&s.ri1[i]);
-        o_r2[k] = ld(&s.ri2[i]);
-        o_r3[k] = ld(&s.ri3[i]);
+    for (int u = 0; u < TPT; u++) {
+        const Own w = own_block<TWC>(g, t, u);
+        const int Wg = o.W0 + w.wl, y = o.y0 + w.yl;
+        nl[u] = w.n;
+        cell[u] = w.n ? l.cell(w.yl, w.j0, w.wl) : 0;
+        if (Wg >= g.ng || y >= g.h) cell[u] = -cell[u];
+        gi[u] = ((int64_t)y * g.K + w.j0) * g.P + Wg;
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) {
+            o_ex[u][k] = o_rc[u][k] = o_rr[u][k] = o_rd[u][k] = o_r0[u][k] = o_r1[u][k] =
+                o_r2[u][k] = o_r3[u][k] = 0;
+            o_ht[u][k] = kInfH;
+            if (cell[u] <= 0 || k >= nl[u]) continue;
+            const int64_t i = gi[u] + (int64_t)k * g.P;
+            o_ex[u][k] = ld(&s.ex[i]);
+            o_ht[u][k] = ld(&s.ht[i]);
+            o_rc[u][k] = ld(&s.rc[i]);
+            o_rr[u][k] = ld(&s.rr[i]);
+            o_rd[u][k] = ld(&s.rd[i]);
+            o_r0[u][k] = ld(&s.ri0[i]);
+            o_r1[u][k] = ld(&s.ri1[i]);
+            o_r2[u][k] = ld(&s.ri2[i]);
+            o_r3[u][k] = ld(&s.ri3[i]);
+        }
     }
     // ... then the shared-memory stores
-    halo_commit(m, true, hr);
+    halo_commit<TWC>(sm, l, true, hr);
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        if (!((tmask >> k) & 1u)) continue;
-        const int p = info_p(inf[k]);
-        m.ex[p] = o_ex[k];
-        m.ht[p] = o_ht[k];
-        if (!((vmask >> k) & 1u)) continue;
-        m.rc[p] = o_rc[k];
-        m.rr[p] = o_rr[k];
-        m.rd[p] = o_rd[k];
-        m.ri0[p] = o_r0[k];
-        m.ri1[p] = o_r1[k];
-        m.ri2[p] = o_r2[k];
-        m.ri3[p] = o_r3[k];
+    for (int u = 0; u < TPT; u++) {
+        int32_t *c = sm + abs(cell[u]);
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) {
+            if (cell[u] == 0 || k >= nl[u]) continue;
+            c[l.at(F_EX, k)] = o_ex[u][k];
+            c[l.at(F_HT, k)] = o_ht[u][k];
+            if (cell[u] < 0) continue;
+            c[l.at(F_RC, k)] = o_rc[u][k];
+            c[l.at(F_RR, k)] = o_rr[u][k];
+            c[l.at(F_RD, k)] = o_rd[u][k];
+            c[l.at(F_I0, k)] = o_r0[u][k];
+            c[l.at(F_I1, k)] = o_r1[u][k];
+            c[l.at(F_I2, k)] = o_r2[u][k];
+            c[l.at(F_I3, k)] = o_r3[u][k];
+        }
     }
-    halo_rest(a, m, o, true, s.ht);
+    halo_rest<TWC>(a, sm, l, o, true, s.ht);
     __syncthreads();
-    int off[kSlots];
+    // the first list
+    const unsigned base = (unsigned)__cvta_generic_to_shared(sm);
+    const unsigned lists = base + 4 * (t.words + t.nblk + 2), nowhere = lists + 4 * t.TN;
+    {
+        unsigned b[TPT][kBlk];
+        int total = 0;
 #pragma unroll
-    for (int q = 0; q < kSlots; q++) off[q] = soff(t, q);
-    int32_t *const sbase = m.ht;                 // field f of the tile at sbase + f * PN
-    const int64_t gstride = s.rr - s.rc;         // global fields are equally spaced
-    // Local iterations, one warp at a time and with no block barrier: each
-    // warp compacts its own active nodes (positive excess, finite height; the
-    // nodes its lanes own) into a warp list of packed positions with ballots,
-    // discharges the list 32 nodes at a time, and goes on to its next
-    // iteration.  Discharges of different warps run concurrently on shared
-    // memory; the lock-free argument that holds between tiles holds between
-    // warps (only a node's own warp lowers its excess, and residuals are
-    // consumed only by an arc's tail).  Every load of a discharge depends only
-    // on the list entry, so they are in flight together.
-    unsigned nb_touch = 0;   // bit 0: left, 1: right, 2: up, 3: down neighbour tile received flow
-    const int lane = threadIdx.x & 31;
-    uint32_t *wl_list = s_wlist[threadIdx.x >> 5];
-    volatile int32_t *vex = m.ex;
-    volatile int32_t *vht = m.ht;
+        for (int u = 0; u < TPT; u++)
+#pragma unroll
+            for (int k = 0; k < kBlk; k++) {
+                b[u][k] = __ballot_sync(0xffffffffu, o_ex[u][k] > 0 && o_ht[u][k] < kInfH);
+                total += __popc(b[u][k]);
+            }
+        int at = 0;
+        if (lane == 0 && total) at = atomicAdd(&s_nodes[0], total);
+        at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+        for (int u = 0; u < TPT; u++)
+#pragma unroll
+            for (int k = 0; k < kBlk; k++) {
+                const int i = at + __popc(b[u][k] & ((1u << lane) - 1u));
+                sts16((b[u][k] >> lane) & 1u ? lists + 2 * i : nowhere, cell[u] + l.at(F_EX, k));
+                at += __popc(b[u][k]);
+            }
+    }
+    const int4 st[4] = {s_slot[4 * (lane & 3)], s_slot[4 * (lane & 3) + 1],
+                        s_slot[4 * (lane & 3) + 2], s_slot[4 * (lane & 3) + 3]};
+    // Local iterations: the warps share out the nodes of the list, and the
+    // iteration ends with a block barrier.  (With a list of its own per warp
+    // and no barrier, the last warp took twice the average.)  While the list
+    // is one discharge's worth, warp 0 goes on by itself, without barriers
+    // (40 % of the iterations).  Discharges run concurrently on shared memory;
+    // the lock-free argument that holds between tiles holds between warps
+    // (only a node's own discharge lowers its excess, and residuals are
+    // consumed only by an arc's tail).
     // Straggler cut: a step ends when its last item does, so a visit still
     // running when nearly all of its step's items are done (all but 1 +
     // min(items / 8, half the grid)) stops after half its local iterations.
     // Its tile keeps its work and is queued for the next round.  Thread 0
-    // reads the step's done count once per iteration and uses it one
-    // iteration later (the load's latency hides behind the iteration).  No
-    // cut without done_ctr (fixed-sweep mode: a round is a full round).
-    unsigned seen = 0;
+    // loads the step's done count every fourth iteration and looks at it two
+    // iterations later (an iteration is shorter than the load).  No cut
+    // without done_ctr (fixed-sweep mode: a round is a full round).
     const unsigned margin = 1 + min(items / 8, gridDim.x / 2);
-    for (int it = 0; it < iters; it++) {
-        if (done_ctr && threadIdx.x == 0) {
-            if (it >= 2 && seen + margin >= items) s_stop = 1;
-            seen = *(volatile const unsigned *)done_ctr;
+    const unsigned counts = (unsigned)__cvta_generic_to_shared(s_nodes);
+    unsigned seen = 0;
+    bool stop = false, shared = false;
+    int it = 0, turn = 0;
+    auto iteration = [&](int i, int first, int n) {
+        if (threadIdx.x == 0) {
+            if (done_ctr && (i & 3) == 0) seen = *(volatile const unsigned *)done_ctr;
+            if (done_ctr && (i & 3) == 2) stop = seen + margin >= items;
+            s_nodes[(i + kLens / 2) % kLens] = 0;
         }
-        if (it >= iters / 2 && __shfl_sync(0xffffffffu, *(volatile int *)&s_stop, 0)) break;
-        int32_t ce[NPT], ch[NPT];
-#pragma unroll
-        for (int k = 0; k < NPT; k++) {
-            const int p = info_p(inf[k]);
-            ce[k] = vex[p];
-            ch[k] = vht[p];
+#pragma unroll 1
+        for (; first < n; first += 8 * W)
+            discharge<TWC>(l, base, lists + 2 * t.TN * (i & 1), first, n, st,
+                           lists + 2 * t.TN * ((i + 1) & 1), counts + 4 * ((i + 1) % kLens),
+                           nowhere);
+    };
+    __syncthreads();
+    while (it < iters) {
+        int n = s_nodes[it % kLens];
+        if (n == 0) break;
+        if (n > 8 || shared) {
+            iteration(it, 8 * warp, n);
+            if (threadIdx.x == 0) s_stop[turn] = stop;
+            __syncthreads();
+            it++;
+            if (it >= iters / 2 && s_stop[turn]) break;
+            turn ^= 1;
+            shared = false;
+        } else {
+            if (warp == 0) {
+                int i = it;
+                do {
+                    iteration(i, 0, n);
+                    __syncwarp();
+                    n = *(volatile int *)&s_nodes[++i % kLens];
+                    if (i >= iters / 2 && __shfl_sync(0xffffffffu, (int)stop, 0)) i = iters;
+                } while (i < iters && n > 0 && n <= 8 && i - it < kLens / 2 - 4);
+                if (lane == 0) s_it = i;
+            }
+            __syncthreads();
+            it = s_it;
+            shared = true;       // (s_it is read before the next barrier)
         }
-        int cnt = 0;
-#pragma unroll
-        for (int k = 0; k < NPT; k++) {
-            const bool act = ((vmask >> k) & 1u) && ce[k] > 0 && ch[k] < kInfH;
-            const unsigned bal = __ballot_sync(0xffffffffu, act);
-            if (act) wl_list[cnt + __popc(bal & ((1u << lane) - 1u))] = inf[k];
-            cnt += __popc(bal);
-        }
-        __syncwarp();
-        if (cnt == 0) continue;
-        for (int li = lane; li < cnt; li += 32) {
-            const uint32_t info = wl_list[li];
-            const int p = info_p(info);
-            const int wl = info_wl(info), yl = info_yl(info), j = info_j(info);
-            const int64_t gin = tile_g0 + (int64_t)yl * g.SY + (int64_t)j * g.P + wl;
-            const unsigned exb = arc_exists(g, o.y0 + yl, j, o.W0 + wl);
-            // all loads issued before any is used (the existing arcs' heights
-            // are read whatever their residual), so they overlap
-            const int32_t e = vex[p];
-            const int32_t hu = vht[p];
-            int32_t rr[kSlots], hv[kSlots];
-#pragma unroll
-            for (int q = 0; q < kSlots; q++) {
-                const bool ex = (exb >> q) & 1u;
-                rr[q] = ex ? smem_residual(m, t, g, p, q) : 0;
-                hv[q] = vht[p + (ex ? off[q] : 0)];
-            }
-            if (e <= 0 || hu >= kInfH) continue;
-            // residual and admissible slots as bit masks (registers only)
-            unsigned resid = 0, adm = 0;
-#pragma unroll
-            for (int q = 0; q < kSlots; q++) {
-                const bool rp = rr[q] > 0;
-                resid |= (unsigned)rp << q;
-                adm |= (unsigned)(rp && hv[q] < hu) << q;
-            }
-            int32_t left = e;
-            // push along the admissible slots, in slot order, until the
-            // excess is gone; a slot's residual is the one loaded above (it
-            // can only have grown since: pushing it is always valid)
-            for (unsigned bits = adm; bits && left > 0; bits &= bits - 1u) {
-                const int q = __ffs(bits) - 1;
-                int32_t r = 0;
-#pragma unroll
-                for (int qq = 0; qq < kSlots; qq++) r = qq == q ? rr[qq] : r;
-                const int32_t d = min(left, r);
-                const SlotTab st = s_slot[q];
-                int32_t *wp = sbase + p + st.a.x;
-                red_add_smem(wp, st.a.z == 0 ? -d : d);
-                const int wl2 = wl + st.b.x, yl2 = yl + st.b.y;
-                if (wl2 < 0 || wl2 >= t.TW || yl2 < 0 || yl2 >= t.TH) {
-                    // the head is a halo node: its excess, and a word stored
-                    // at it, change in global memory at once
-                    if (st.a.z == 1) red_add_gmem(s.rc + st.b.z * gstride + gin + st.b.w, d);
-                    red_add_gmem(s.ex + gin + st.c.x, d);
-                    nb_touch |= wl2 < 0 ? 1u : wl2 >= t.TW ? 2u : yl2 < 0 ? 4u : 8u;
-                } else {
-                    red_add_smem(sbase + p + st.a.y, d);
-                }
-                left -= d;
-            }
-            if (left != e) red_add_smem(&m.ex[p], left - e);
-            if (left > 0) {
-                // every admissible slot is saturated: relabel over the others
-                const unsigned rest = resid & ~adm;
-                int32_t hmin = kInfH;
-#pragma unroll
-                for (int q = 0; q < kSlots; q++)
-                    if ((rest >> q) & 1u) hmin = min(hmin, hv[q]);
-                vht[p] = hmin >= kInfH - 1 ? kInfH : hmin + 1;
-            }
-        }
-        __syncwarp();
     }
     __syncthreads();
     // write back own nodes as deltas (other tiles may have updated the same
     // words through global atomics meanwhile); note whether work is left
     int still = 0;
 #pragma unroll
-    for (int k = 0; k < NPT; k++) {
-        if (!((vmask >> k) & 1u)) continue;
-        const uint32_t info = inf[k];
-        const int p = info_p(info);
-        const int64_t i = tile_g0 + (int64_t)info_yl(info) * g.SY +
-                          (int64_t)info_j(info) * g.P + info_wl(info);
-        int32_t v;
-        if ((v = m.ex[p] - o_ex[k])) atomicAdd(&s.ex[i], v);
-        // the data-arc residual is the one word that can grow without a bound
-        // of its own (flow pushed back down the infinite reverse arc); only
-        // this tile changes it (the chain stays inside the tile)
-        overflow |= m.rc[p] > kCapLimit || m.rc[p] < 0;
-        if ((v = m.rc[p] - o_rc[k])) atomicAdd(&s.rc[i], v);
-        if ((v = m.rr[p] - o_rr[k])) atomicAdd(&s.rr[i], v);
-        if ((v = m.rd[p] - o_rd[k])) atomicAdd(&s.rd[i], v);
-        if ((v = m.ri0[p] - o_r0[k])) atomicAdd(&s.ri0[i], v);
-        if ((v = m.ri1[p] - o_r1[k])) atomicAdd(&s.ri1[i], v);
-        if ((v = m.ri2[p] - o_r2[k])) atomicAdd(&s.ri2[i], v);
-        if ((v = m.ri3[p] - o_r3[k])) atomicAdd(&s.ri3[i], v);
-        if (m.ht[p] != o_ht[k]) __stcg(&s.ht[i], m.ht[p]);
-        still |= m.ex[p] > 0 && m.ht[p] < kInfH;
+    for (int u = 0; u < TPT; u++) {
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) {
+            if (cell[u] <= 0 || k >= nl[u]) continue;
+            const int32_t *c = sm + cell[u] + l.at(0, k);
+            const int64_t i = gi[u] + (int64_t)k * g.P;
+            const int32_t ex = c[l.at(F_EX)], ht = c[l.at(F_HT)], rc = c[l.at(F_RC)];
+            // the data-arc residual is the one word that can grow without a
+            // bound of its own (flow pushed back down the infinite reverse
+            // arc); only this tile changes it (the chain stays inside the tile)
+            overflow |= rc > kCapLimit || rc < 0;
+            red_add_nz(&s.ex[i], ex - o_ex[u][k]);
+            red_add_nz(&s.rc[i], rc - o_rc[u][k]);
+            red_add_nz(&s.rr[i], c[l.at(F_RR)] - o_rr[u][k]);
+            red_add_nz(&s.rd[i], c[l.at(F_RD)] - o_rd[u][k]);
+            red_add_nz(&s.ri0[i], c[l.at(F_I0)] - o_r0[u][k]);
+            red_add_nz(&s.ri1[i], c[l.at(F_I1)] - o_r1[u][k]);
+            red_add_nz(&s.ri2[i], c[l.at(F_I2)] - o_r2[u][k]);
+            red_add_nz(&s.ri3[i], c[l.at(F_I3)] - o_r3[u][k]);
+            stg_if(ht != o_ht[u][k], &s.ht[i], ht);
+            still |= ex > 0 && ht < kInfH;
+        }
+    }
+    // flow pushed into halo nodes: their excess, and the words stored at them
+    unsigned bits = (still ? 16u : 0u) | (overflow ? 32u : 0u);
+    const int cells = halo_cells<TWC>(g, t);
+    for (int n = threadIdx.x; n < cells; n += blockDim.x) {
+        int hc, kind;
+        int64_t gh;
+        bool in;
+        halo_cell<TWC>(g, t, l, o, n, hc, gh, in, kind);
+        const int32_t *c = sm + hc;
+        const int32_t v = c[l.at(F_EX)] - 1;
+        if (v == 0) continue;
+        red_add_gmem(&s.ex[gh], v);
+        bits |= 1u << kind;
+        const int64_t gs = s.rr - s.rc;          // global fields are equally spaced
+        int32_t d = c[l.at(halo_f1(kind))] - c[l.at(F_KEEP1)];
+        if (d) red_add_gmem(s.rc + (halo_f1(kind) - F_RC) * gs + gh, d);
+        if (halo_f2(kind) >= 0) {
+            d = c[l.at(halo_f2(kind))] - c[l.at(halo_k2(kind))];
+            if (d) red_add_gmem(s.rc + (halo_f2(kind) - F_RC) * gs + gh, d);
+        }
     }
     // one barrier for the tile's flags: bits 0-3 neighbour tiles that received
-    // flow, bit 4 work left in this tile
-    const unsigned wbits = __reduce_or_sync(0xffffffffu, nb_touch | (still ? 16u : 0u));
-    if ((threadIdx.x & 31) == 0 && wbits) atomicOr(&s_touch, wbits);
+    // flow (left, right, up, down), bit 4 work left in this tile, bit 5 overflow
+    bits = __reduce_or_sync(0xffffffffu, bits);
+    if (lane == 0 && bits) atomicOr(&s_touch, bits);
     __syncthreads();
     const unsigned touch = s_touch;
-    const bool still_any = (touch & 16u) != 0;
     if (threadIdx.x < 4 && (touch >> threadIdx.x & 1u)) {
         const int nb = side_tile(t, o, tile, threadIdx.x);
         if (nb >= 0) enqueue(act_next, list_next, count_next, nb);
     }
-    if (threadIdx.x == 4 && still_any) enqueue(act_next, list_next, count_next, tile);
-    __syncthreads();
+    if (threadIdx.x == 4 && (touch & 16u)) enqueue(act_next, list_next, count_next, tile);
+    overflow = (touch & 32u) != 0;
 }
 
 // ------------------------------------------------------- the solve loop ---
@@ -1069,21 +1198,23 @@ struct PairState {
 // Per-pair control words of a launch.  claim packs the current step's queue
 // slot (step mod 3), its number of items and the next item (24 bits each):
 // one atomic add both claims an item and tells where its step's queue is.
+// The words that idle blocks poll (claim), that running visits poll (done),
+// that visits add to, and the state lie in cache lines of their own.
 struct PairCtl {
-    unsigned long long claim;
-    unsigned int done;      // items of the current step completed
-    unsigned int step;      // current step
-    long long red[3][4];    // per-step sums (slot = step mod 3)
-    int32_t qcount[3];      // queued tiles per step slot
-    int32_t pad;
-    PairState st;           // written only by the block that advances the pair
+    alignas(128) unsigned long long claim;
+    alignas(128) unsigned int done;   // items of the current step completed
+    alignas(128) long long red[3][4]; // per-step sums (slot = step mod 3)
+    int32_t qcount[3];                // queued tiles per step slot
+    unsigned int step;                // current step
+    alignas(128) PairState st;        // written only by the block that advances the pair
 };
 
 constexpr unsigned kItemMask = 0xffffffu;
 // An idle block gives up after this long unless the options set a limit.
 constexpr unsigned long long kDefaultIdleLimitNs = 60ull * 1000 * 1000 * 1000;
 
-static_assert(sizeof(PairState) % 8 == 0, "PairState is copied in 8-byte words");
+constexpr int kStateWords = sizeof(PairState) / 8;
+static_assert(sizeof(PairState) % 8 == 0 && kStateWords <= 28, "a warp copies PairState, a word a lane");
 
 // Copy of a pair's state as other SMs wrote it (L2-coherent loads).
 __device__ __forceinline__ void load_state(PairState *dst, const PairState *src) {
@@ -1292,60 +1423,222 @@ __device__ void pair_results(const BatchArgs &B, const PairState &st, const Solv
     if (status != GS_OK) atomicCAS(a.status, GS_OK, status);
 }
 
-// End of a pair's step (one thread, after every item completed): advance the
+// End of a pair's step (one warp, after every item completed): advance the
 // state machine -- through any steps that have no items -- and publish the
-// next step's claim word, or count the pair finished.
-__device__ void end_step(const BatchArgs &B, int p, int slot) {
+// next step's claim word, or count the pair finished.  s_st holds the pair's
+// state, unchanged since the step began.
+__device__ __forceinline__ void end_step(const BatchArgs &B, int p, int slot, PairState &s_st) {
     PairCtl *c = B.ctl + p;
     const SolveArgs &a = B.pair[p];
-    // the step's sums, its number, the pair's state and the queue the step
-    // filled for the next one, loaded together (the caller's acquire on the
-    // done count orders them after every item's writes)
+    const int lane = threadIdx.x & 31;
+    // the step's sums, the queue the step filled for the next one and its
+    // number, loaded together (the caller's acquire on the done count orders
+    // them after every item's writes)
+    long long mine = 0;
+    if (lane < 4) mine = *(volatile long long *)&c->red[slot][lane];
+    else if (lane == 4) mine = *(volatile int32_t *)&c->qcount[(slot + 1) % 3];
+    else if (lane == 5) mine = *(volatile unsigned *)&c->step;
     long long v0[4];
-    for (int k = 0; k < 4; k++) v0[k] = *(volatile long long *)&c->red[slot][k];
-    const int32_t q0 = *(volatile int32_t *)&c->qcount[(slot + 1) % 3];
-    unsigned step = *(volatile unsigned *)&c->step;
-    PairState st;
-    load_state(&st, &c->st);
-    bool first = true;
+#pragma unroll
+    for (int k = 0; k < 4; k++) v0[k] = __shfl_sync(0xffffffffu, mine, k);
+    const int32_t q0 = (int32_t)__shfl_sync(0xffffffffu, mine, 4);
+    unsigned step = (unsigned)__shfl_sync(0xffffffffu, mine, 5);
     unsigned items = 0;
-    const unsigned long long t_now = now_ns();
-    if (st.phase == PH_SWEEP) st.ns_sweep += (long long)(t_now - st.t_step);
-    else st.ns_relabel += (long long)(t_now - st.t_step);
-    st.t_step = t_now;
-    for (;;) {
-        long long v[4];
-        const bool pre = first && step % 3 == (unsigned)slot;   // the prefetched words apply
-        if (pre)
-            for (int k = 0; k < 4; k++) v[k] = v0[k];
-        else
-            for (int k = 0; k < 4; k++) v[k] = *(volatile long long *)&c->red[step % 3][k];
-        first = false;
-        advance(st, a, v, B.extract);
-        const unsigned next = step + 1;
-        for (int k = 0; k < 4; k++) c->red[next % 3][k] = 0;
-        c->qcount[(next + 1) % 3] = 0;
-        items = st.phase == PH_DONE ? 0u
-                : (pre && queued(st)) ? (unsigned)q0
-                                      : step_items(st, a, c, next);
-        step = next;
-        if (st.phase == PH_DONE || items > 0) break;
+    bool finished = false;
+    if (lane == 0) {
+        PairState st = s_st;
+        bool first = true;
+        const unsigned long long t_now = now_ns();
+        if (st.phase == PH_SWEEP) st.ns_sweep += (long long)(t_now - st.t_step);
+        else st.ns_relabel += (long long)(t_now - st.t_step);
+        st.t_step = t_now;
+        for (;;) {
+            long long v[4];
+            const bool pre = first && step % 3 == (unsigned)slot;   // the prefetched words apply
+            if (pre)
+                for (int k = 0; k < 4; k++) v[k] = v0[k];
+            else
+                for (int k = 0; k < 4; k++) v[k] = *(volatile long long *)&c->red[step % 3][k];
+            first = false;
+            advance(st, a, v, B.extract);
+            const unsigned next = step + 1;
+            for (int k = 0; k < 4; k++) c->red[next % 3][k] = 0;
+            c->qcount[(next + 1) % 3] = 0;
+            items = st.phase == PH_DONE ? 0u
+                    : (pre && queued(st)) ? (unsigned)q0
+                                          : step_items(st, a, c, next);
+            step = next;
+            if (st.phase == PH_DONE || items > 0) break;
+        }
+        c->done = 0;
+        c->step = step;
+        s_st = st;
+        finished = st.phase == PH_DONE;
+        if (finished) pair_results(B, st, a, st.status);
     }
-    c->st = st;
-    c->done = 0;
-    c->step = step;
-    if (st.phase == PH_DONE) pair_results(B, st, a, st.status);
-    atom_exch_release(&c->claim, pack_claim(step, items, 0));
-    if (st.phase == PH_DONE) atomicAdd(&B.bar->active, 1);
+    __syncwarp();
+    if (lane < kStateWords) ((long long *)&c->st)[lane] = ((const long long *)&s_st)[lane];
+    __syncwarp();
+    if (lane == 0) {
+        atom_exch_release(&c->claim, pack_claim(step, items, 0));
+        if (finished) atomicAdd(&B.bar->active, 1);
+    }
 }
 
-template <int NPT, int BT>
-__global__ void __launch_bounds__(BT, BT == 256 ? 2 : 1) k_batch(const __grid_constant__ BatchArgs B) {
+// The item a block works on.
+struct Item {
+    int p, tile, slot;      // pair, tile, queue slot of the step (tile < 0: the launch is over)
+    unsigned items, idx;    // items of the step, this one's number
+};
+
+// Sums of a completed item (active nodes or worked tiles, changes, visits, overflow).
+struct ItemSums {
+    long long a, b, c;
+    int ovf;
+};
+
+// Complete the block's item `it` (it.tile >= 0: a visit with sums v) and claim
+// the next one that has work, into it and s_st (warp 0; the caller's block
+// barrier hands them to the other warps).
+// The atomic that claims the next item of the same step goes out before the
+// one that counts the completed item, so the two round trips overlap; the
+// words a claimed item needs are loaded by one lane each.
+__device__ __forceinline__ void next_item(const BatchArgs &B, Item &it, const ItemSums &v0,
+                                          PairState &s_st) {
+    const int lane = threadIdx.x & 31;
+    ItemSums v = v0;
+    bool finish = it.tile >= 0;
+    for (;;) {
+        unsigned long long w = 0;
+        bool got = false;
+        if (finish) {
+            PairCtl *c = B.ctl + it.p;
+            // (only with more items left than blocks: near the end of a step
+            // its completion must not wait for a claim that may find nothing)
+            const bool more = it.idx + gridDim.x < it.items;
+            bool last = false;
+            if (lane == 0) {
+                long long *rp = c->red[it.slot];
+                if (v.a) atomicAdd((unsigned long long *)&rp[0], (unsigned long long)v.a);
+                if (v.b) atomicAdd((unsigned long long *)&rp[1], (unsigned long long)v.b);
+                if (v.c) atomicAdd((unsigned long long *)&rp[2], (unsigned long long)v.c);
+                if (v.ovf) atomicAdd((unsigned long long *)&rp[3], 1ull);
+                if (more) w = atom_add_relaxed(&c->claim, 1ull);
+                // a release (the item's writes before it) and an acquire (every
+                // item's writes, and what the claim above names, after it); the
+                // step cannot end before this item does
+                last = atom_add_acq_rel(&c->done, 1u) + 1u == it.items;
+            }
+            w = __shfl_sync(0xffffffffu, w, 0);
+            if (__shfl_sync(0xffffffffu, (int)last, 0)) end_step(B, it.p, it.slot, s_st);
+            got = more && (w & kItemMask) < ((w >> 24) & kItemMask);
+        }
+        int p = it.p, over = 0;
+        if (!got && lane == 0) {
+            // poll the pairs' claim words; idle polling backs off to 256 ns
+            const unsigned long long t0 = now_ns();
+            for (int spin = 0; !got && !over; spin++) {
+                if (aborted(B.bar) || *(volatile int32_t *)&B.bar->active >= B.n) {
+                    over = 1;
+                    break;
+                }
+                for (int k = 0; k < B.n && !got; k++) {
+                    p = (int)((blockIdx.x + k) % B.n);
+                    PairCtl *c = B.ctl + p;
+                    w = *(volatile unsigned long long *)&c->claim;
+                    if ((w & kItemMask) >= ((w >> 24) & kItemMask)) continue;
+                    w = atom_add_acquire(&c->claim, 1ull);
+                    got = (w & kItemMask) < ((w >> 24) & kItemMask);
+                }
+                if (got) break;
+                if (now_ns() - t0 > B.idle_limit_ns) {
+                    atomicExch(&B.bar->abort, 1);
+                    over = 1;
+                    break;
+                }
+                __nanosleep(32u << min(spin, 3));
+            }
+        }
+        p = __shfl_sync(0xffffffffu, p, 0);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        it.tile = -1;
+        if (__shfl_sync(0xffffffffu, over, 0)) return;
+        it.p = p;
+        it.slot = (int)((w >> 48) & 3u);
+        it.items = (unsigned)((w >> 24) & kItemMask);
+        it.idx = (unsigned)(w & kItemMask);
+        // everything the item needs, loaded together: the pair's state, both
+        // ways the item may name its tile (the queued tile at this slot, or
+        // tile idx with its count of active nodes), and the abort flag
+        const SolveArgs &a = B.pair[p];
+        const PairCtl *c = B.ctl + p;
+        int32_t x = 0;
+        if (lane < kStateWords)
+            ((long long *)&s_st)[lane] = __ldcg((const long long *)&c->st + lane);
+        else if (lane == 29) x = ld(&a.tile_list[it.slot * a.t.T + it.idx]);
+        else if (lane == 30) x = ld(&a.tile_cnt[it.idx]);
+        else if (lane == 31) x = *(volatile int32_t *)&B.bar->abort;
+        __syncwarp();
+        const int qt = __shfl_sync(0xffffffffu, x, 29), tc = __shfl_sync(0xffffffffu, x, 30);
+        if (__shfl_sync(0xffffffffu, x, 31)) return;      // aborted: leave (tile stays -1)
+        it.tile = queued(s_st) ? qt : (int)it.idx;
+        if (queued(s_st) || s_st.phase != PH_SWEEP || tc > 0) return;
+        // nothing to sweep in this tile: complete at once
+        v.a = v.b = v.c = 0;
+        v.ovf = 0;
+        finish = true;
+    }
+}
+
+// One item of a step.
+struct Visit {
+    int tile, next, T;
+    unsigned items;
+};
+
+template <int TPT, int TWC>
+__device__ __forceinline__ void visit_tile(const SolveArgs &a, PairCtl *c, const PairState &st,
+                                           const Visit &v, int32_t *sm, ItemSums &sums) {
+    int32_t *list_next = a.tile_list + v.next * v.T;
+    int32_t *count_next = &c->qcount[v.next];
+    const int tile = v.tile;
+    if (st.phase == PH_INIT) {
+        if (threadIdx.x == 0) {
+            __stcg(&a.tile_dirty[tile], 0);
+            __stcg(&a.tile_dirty[v.T + tile], 0);
+            __stcg(&a.tile_act[tile], 0);
+            __stcg(&a.tile_act[v.T + tile], 0);
+        }
+        sums.a = relabel_init_tile<TPT, TWC>(a, sm, tile);
+        sums.c = 1;
+    } else if (st.phase == PH_PASS) {
+        const int pass = st.pass;
+        int32_t *dcur = a.tile_dirty + (pass & 1) * v.T;
+        int32_t *dnext = a.tile_dirty + ((pass + 1) & 1) * v.T;
+        if (pass > 1 && threadIdx.x == 0) __stcg(&dcur[tile], 0);
+        int ch = 0;
+        sums.a = relabel_pass_tile<TPT, TWC>(a, sm, tile, ch, dnext, list_next, count_next, &c->done,
+                                             v.items);
+        sums.b = ch;
+        sums.c = 1;
+    } else {   // PH_SWEEP
+        const int cur = (int)(st.round & 1);
+        if (threadIdx.x == 0) __stcg(&a.tile_act[cur * v.T + tile], 0);
+        const int iters = st.tail ? a.tail_iters : a.local_iters;
+        const unsigned *done_ctr = a.mode == GS_MODE_FIXED_SWEEPS ? nullptr : &c->done;
+        sweep_tile<TPT, TWC>(a, sm, tile, cur, iters, sums.ovf, list_next, count_next, done_ctr,
+                             v.items);
+        sums.a = 1;
+    }
+}
+
+// TPT: blocks of own nodes per thread, the most any pair of the launch needs.
+// Blocks of 256 or 512 threads; 128 registers a thread leave room for two or
+// one of them per SM.
+template <int TPT>
+__global__ void __launch_bounds__(kTileThreads, 1) k_batch(const __grid_constant__ BatchArgs B) {
     extern __shared__ int32_t smem[];
-    __shared__ uint32_t s_wlist[BT / 32][8 * 32];   // the sweep's per-warp active lists
-    // pair, item, queue slot of the step, exit flag, items of the step, the
-    // queued tile at the item (speculative), the item's tile count (speculative)
-    __shared__ int s_claim[7];
+    __shared__ Item s_item;
     __shared__ PairState s_st;
     int tables_for = -1;           // pair whose tile-shape tables the block holds
     // block 0 starts every pair and publishes its first step
@@ -1379,132 +1672,46 @@ __global__ void __launch_bounds__(BT, BT == 256 ? 2 : 1) k_batch(const __grid_co
             if (st.phase == PH_DONE) atomicAdd(&B.bar->active, 1);
         }
     }
+    Item it = {0, -1, 0, 0, 0};
+    ItemSums sums = {0, 0, 0, 0};
     for (;;) {
-        // claim an item of any pair (thread 0); idle polling backs off to 256 ns
-        if (threadIdx.x == 0) {
-            const unsigned long long t0 = now_ns();
-            int got = 0;
-            for (int spin = 0; !got; spin++) {
-                if (aborted(B.bar) || *(volatile int32_t *)&B.bar->active >= B.n) {
-                    s_claim[3] = 1;
-                    break;
-                }
-                for (int k = 0; k < B.n && !got; k++) {
-                    const int p = (int)((blockIdx.x + k) % B.n);
-                    PairCtl *c = B.ctl + p;
-                    const unsigned long long w0 = *(volatile unsigned long long *)&c->claim;
-                    if ((w0 & kItemMask) >= ((w0 >> 24) & kItemMask)) continue;
-                    const unsigned long long w = atom_add_acquire(&c->claim, 1ull);
-                    const unsigned items = (unsigned)((w >> 24) & kItemMask);
-                    const unsigned idx = (unsigned)(w & kItemMask);
-                    if (idx >= items) continue;
-                    // everything the item needs, loaded together: the pair's
-                    // state, and both ways the item may name its tile (the
-                    // queued tile at this slot, or tile idx with its count)
-                    const int sl = (int)((w >> 48) & 3u);
-                    const SolveArgs &ap = B.pair[p];
-                    const int32_t qt = ld(&ap.tile_list[sl * ap.t.T + idx]);
-                    const int32_t tc = ld(&ap.tile_cnt[idx]);
-                    load_state(&s_st, &c->st);
-                    s_claim[0] = p;
-                    s_claim[1] = (int)idx;
-                    s_claim[2] = sl;
-                    s_claim[3] = 0;
-                    s_claim[4] = (int)items;
-                    s_claim[5] = qt;
-                    s_claim[6] = tc;
-                    got = 1;
-                }
-                if (!got) {
-                    if (now_ns() - t0 > B.idle_limit_ns) {
-                        atomicExch(&B.bar->abort, 1);
-                        s_claim[3] = 1;
-                        break;
-                    }
-                    __nanosleep(32u << min(spin, 3));
-                }
-            }
+        if (threadIdx.x < 32) {
+            next_item(B, it, sums, s_st);
+            if (threadIdx.x == 0) s_item = it;
         }
         __syncthreads();
-        if (s_claim[3]) break;
-        const int pr = s_claim[0];
-        const int slot = s_claim[2], next = (slot + 1) % 3;
-        PairCtl *c = B.ctl + pr;
-        const SolveArgs &a = B.pair[pr];
-        if (pr != tables_for) {      // uniform: every thread read the same claim
-            build_tables(a);
-            tables_for = pr;
+        it = s_item;
+        if (it.tile < 0) break;
+        PairCtl *c = B.ctl + it.p;
+        const SolveArgs &a = B.pair[it.p];
+        if (it.p != tables_for) {    // uniform: every thread read the same item
+            build_tables(a, smem);
+            tables_for = it.p;
             __syncthreads();
         }
-        const int phase = s_st.phase;
-        const int T = a.t.T;
-        const TileSmem m = tile_smem(smem, a.t.PN);
-        int32_t *list_next = a.tile_list + next * T;
-        int32_t *count_next = &c->qcount[next];
-        const int tile = queued(s_st) ? s_claim[5]
-                         : (phase == PH_SWEEP && s_claim[6] <= 0) ? -1   // nothing to sweep
-                                                                   : s_claim[1];
-        long long va = 0, vb = 0, vc = 0;
-        int ovf = 0;
-        if (tile >= 0) {
-            if (phase == PH_INIT) {
-                // a pair whose tiles need 4 nodes per thread runs the
-                // 4-node code also when the launch is sized for 8
-                va = (NPT == 8 && a.npt == 4) ? relabel_init_tile<4>(a, m, tile)
-                                              : relabel_init_tile<NPT>(a, m, tile);
-                vc = 1;
-                if (threadIdx.x == 0) {
-                    __stcg(&a.tile_dirty[tile], 0);
-                    __stcg(&a.tile_dirty[T + tile], 0);
-                    __stcg(&a.tile_act[tile], 0);
-                    __stcg(&a.tile_act[T + tile], 0);
-                }
-            } else if (phase == PH_PASS) {
-                const int pass = s_st.pass;
-                int32_t *dcur = a.tile_dirty + (pass & 1) * T;
-                int32_t *dnext = a.tile_dirty + ((pass + 1) & 1) * T;
-                if (pass > 1 && threadIdx.x == 0) __stcg(&dcur[tile], 0);
-                int ch = 0;
-                va = (NPT == 8 && a.npt == 4)
-                         ? relabel_pass_tile<4>(a, m, tile, ch, dnext, list_next, count_next,
-                                                &c->done, (unsigned)s_claim[4])
-                         : relabel_pass_tile<NPT>(a, m, tile, ch, dnext, list_next, count_next,
-                                                  &c->done, (unsigned)s_claim[4]);
-                vb = ch;
-                vc = 1;
-            } else if (phase == PH_SWEEP) {
-                const int cur = (int)(s_st.round & 1);
-                if (threadIdx.x == 0) __stcg(&a.tile_act[cur * T + tile], 0);
-                const int iters = s_st.tail ? a.tail_iters : a.local_iters;
-                const unsigned *done_ctr = a.mode == GS_MODE_FIXED_SWEEPS ? nullptr : &c->done;
-                if (NPT == 8 && a.npt == 4)
-                    sweep_tile<4, BT>(a, m, tile, cur, iters, ovf, list_next, count_next, done_ctr,
-                                      (unsigned)s_claim[4], s_wlist);
-                else
-                    sweep_tile<NPT, BT>(a, m, tile, cur, iters, ovf, list_next, count_next,
-                                        done_ctr, (unsigned)s_claim[4], s_wlist);
-                ovf = __syncthreads_or(ovf);
-                va = 1;
-            } else {   // PH_LABELS
-                int bad = 0;
-                va = labels_tile(a, tile, s_st.ht_labels ? a.s.ht : a.hgt, bad);
-                vb = bad;
+        sums = {0, 0, 0, 0};
+        // (a visit has a block barrier after its last look at s_item and s_st,
+        // and ends with warp 0's queueing)
+        if (s_st.phase != PH_LABELS) {
+            // the visit's code for this tile width, and a pair whose tiles
+            // need one block per thread runs that code also when the launch is
+            // sized for two
+            const Visit v = {it.tile, (it.slot + 1) % 3, a.t.T, it.items};
+            if (TPT == 2 && a.tpt == 1) {
+                if (a.t.TW == 8) visit_tile<1, 8>(a, c, s_st, v, smem, sums);
+                else if (a.t.TW == 16) visit_tile<1, 16>(a, c, s_st, v, smem, sums);
+                else visit_tile<1, 0>(a, c, s_st, v, smem, sums);
+            } else {
+                if (a.t.TW == 8) visit_tile<TPT, 8>(a, c, s_st, v, smem, sums);
+                else if (a.t.TW == 16) visit_tile<TPT, 16>(a, c, s_st, v, smem, sums);
+                else visit_tile<TPT, 0>(a, c, s_st, v, smem, sums);
             }
+        } else {
+            int bad = 0;
+            sums.a = labels_tile(a, it.tile, s_st.ht_labels ? a.s.ht : a.hgt, bad);
+            sums.b = bad;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            long long *rp = c->red[slot];
-            if (va) atomicAdd((unsigned long long *)&rp[0], (unsigned long long)va);
-            if (vb) atomicAdd((unsigned long long *)&rp[1], (unsigned long long)vb);
-            if (vc) atomicAdd((unsigned long long *)&rp[2], (unsigned long long)vc);
-            if (ovf) atomicAdd((unsigned long long *)&rp[3], 1ull);
-            // the step's item count, as claimed (the step cannot end before
-            // this item does); the count is a release (the item's writes
-            // before it) and an acquire (every item's writes after it)
-            const unsigned total = (unsigned)s_claim[4];
-            if (atom_add_acq_rel(&c->done, 1u) + 1u == total) end_step(B, pr, slot);
-        }
-        __syncthreads();
+        __syncwarp();
     }
     // pairs still running when the launch gave up
     if (blockIdx.x == 0 && aborted(B.bar)) {
@@ -1519,18 +1726,40 @@ __global__ void __launch_bounds__(BT, BT == 256 ? 2 : 1) k_batch(const __grid_co
 
 // ------------------------------------------------------------ host side ---
 
-// Tile shape: whole chains (all K layers), TW sites x TH rows.  The shared
-// memory holds 9 int32 fields over the tile and a one-site halo; at most 8
-// nodes per thread (4 preferred).  Wider tiles first (coalesced rows of 32
-// sites), then the tallest that fits up to TH = 4.
-static bool pick_tile(const Geom &g, TileGeom &t, int &npt, size_t &smem, int want_w = 0,
-                      int want_h = 0, int bt = kTileThreads) {
-    // dynamic shared memory of a tile; with the kernel's ~34 KB of static
-    // shared arrays it must stay under the 227 KB a block may opt in to.  With
-    // 256-thread blocks the library's own choice first tries to keep two tiles
-    // within an SM (long chains fall back to one block per SM).
-    const size_t budgets[2] = {(bt == 256 && !want_w) ? size_t(80 * 1024) : size_t(180 * 1024),
-                               size_t(180 * 1024)};
+// Shared-memory conflicts of the first warp's lanes (their blocks' cells) for a
+// row stride: the largest number of lanes on one bank.
+static int bank_conflicts(int TW, int S, int SJ, int sy) {
+    int hits[32] = {}, worst = 0;
+    for (int n = 0; n < 32; n++) {
+        const int site = n % S;
+        const int w = (site / TW) * sy + (n / S) * kBlk * 9 * SJ + site % TW;
+        worst = std::max(worst, ++hits[w & 31]);
+    }
+    return worst;
+}
+
+// Bytes of a tile's nine fields over its nodes and a one-site halo, rows padded
+// to TW (mod 32) where a warp takes whole rows: the size that the shape rules
+// (and gs_tile_info) go by.  0: never a tile.
+static size_t field_bytes(const Geom &g, int TW, int TH, int bt) {
+    const int64_t TN = (int64_t)TH * g.K * TW;
+    if (TN > 8 * bt || TN > 4096 || g.K >= 2048) return 0;
+    int row = g.K * (TW + 2);
+    if (TH % (32 / TW) == 0) row += ((TW - row) % 32 + 32) % 32;
+    const int64_t cells = (int64_t)(TH + 2) * row;
+    return cells < 8192 ? 9 * cells * sizeof(int32_t) : 0;
+}
+
+// Tile shape: whole chains (all K layers), TW sites x TH rows, the nine fields
+// within 180 KB; one block of kBlk layers per thread, or two.  The library's
+// own choice prefers one, and with 256-thread blocks fields within 80 KB, so
+// that two tiles fit an SM (long chains fall back to one).  A tile takes up to
+// 15 % more shared memory than its fields (the padding between rows, the lists
+// of active nodes), which stays within a block's 227 KB.  `fields` returns
+// field_bytes of the shape, `smem` what the kernel needs.
+static bool pick_tile(const Geom &g, TileGeom &t, int &tpt, size_t &smem, int want_w = 0,
+                      int want_h = 0, int bt = kTileThreads, size_t *fields = nullptr) {
+    const size_t budgets[2] = {(bt == 256 && !want_w ? 80 : 180) * size_t(1024), 180 * 1024};
     // more sites first, squarer first among equals: a breadth-first path then
     // crosses fewer tile borders (measured: 8x8 beats 16x4 at 31 depth layers,
     // 8x4 beats 16x2 at 47)
@@ -1543,63 +1772,58 @@ static bool pick_tile(const Geom &g, TileGeom &t, int &npt, size_t &smem, int wa
             return false;
     }
     for (int pass = 0; pass < 4; pass++) {
-        const size_t budget = budgets[pass / 2];
-        const int max_nodes = (pass % 2 == 0 ? 4 : 8) * bt;
         for (int ci = 0; ci < (want_w ? 1 : (int)(sizeof(cand) / sizeof(cand[0]))); ci++) {
             const int TW = want_w ? want_w : cand[ci][0], TH = want_w ? want_h : cand[ci][1];
-            const int TN = TH * g.K * TW;
-            // Bank-conflict-free placement: a warp takes the same TW sites in
-            // R = 32 / TW consecutive rows of sites (same layer), and the row
-            // stride is padded to TW (mod 32), so its 32 lanes touch 32
-            // different banks in every access of a visit (two rows of 16
-            // sites one layer apart, 18 words apart, shared two banks).
-            // Needs TH a multiple of R.
-            const int R = (TW <= 32 && TH % (32 / TW) == 0) ? 32 / TW : 0;
-            int SYs = g.K * (TW + 2);
-            if (R) SYs += ((TW - SYs) % 32 + 32) % 32;
-            const int PN = (TH + 2) * SYs;
-            const size_t bytes = 9 * (size_t)PN * sizeof(int32_t);
-            // the packed node info holds shared indices below 8192 and depth
-            // layers below 2048
-            if (TN > max_nodes || TN > kMaxTileNodes || bytes > budget || PN >= 8192 ||
-                g.K >= 2048)
-                continue;
+            const size_t fb = field_bytes(g, TW, TH, bt);
+            if (!fb || fb > budgets[pass / 2]) continue;
+            const int per_thread = pass % 2 == 0 ? 1 : 2;
+            const int S = TW * TH, nblk = (g.K + kBlk - 1) / kBlk, SJ = TW + 2;
+            if (nblk * S > per_thread * bt) continue;
+            const int row = 9 * (g.K + 1) * SJ;
+            int pad = 0;
+            for (int x = 1; x < 32; x++)
+                if (bank_conflicts(TW, S, SJ, row + x) < bank_conflicts(TW, S, SJ, row + pad))
+                    pad = x;
+            const int SYs = row + pad;
+            const int words = (TH + 2) * SYs + kBlk * 9 * SJ;
+            const int TN = S * g.K;
+            const size_t bytes = (size_t)(words + nblk + 2 + TN + 1) * sizeof(int32_t);
+            // (a list entry is a cell's 16-bit offset: 224 KB are 57344 words)
+            if (bytes > 224 * 1024) continue;
             t.TW = TW;
             t.TH = TH;
-            t.PW = TW + 2;
-            t.SJ = t.PW;
+            t.SJ = SJ;
             t.SYs = SYs;
-            t.PN = PN;
+            t.words = words;
+            t.S = S;
+            t.nblk = nblk;
             t.TN = TN;
-            t.R = R;
-            // a multiplier near 0.618 M coprime with M: the groups a thread
-            // holds (32 x 16 nodes apart) map to spread-out parts of the tile,
-            // so a cluster of active nodes falls on many warps, not on one
-            t.spread = 1;
-            if (R) {
-                const int M = TN / 32;
-                for (int a = (int)(0.618 * M); a < 2 * M + 2; a++) {
-                    int x = a, y = M;
-                    while (y) {
-                        const int r = x % y;
-                        x = y;
-                        y = r;
-                    }
-                    if (a >= 1 && x == 1) {
-                        t.spread = a % M == 0 ? 1 : a;
-                        break;
-                    }
-                }
-            }
+            t.rTH = TH == 1 ? 0u : (unsigned)((0x100000000ull + TH - 1) / TH);
+            t.rS = (unsigned)((0x100000000ull + S - 1) / S);
             t.tiles_w = (g.ng + TW - 1) / TW;
             t.tiles_h = (g.h + TH - 1) / TH;
             t.T = t.tiles_w * t.tiles_h;
-            npt = pass % 2 == 0 ? 4 : 8;
+            tpt = per_thread;
             smem = bytes;
+            if (fields) *fields = fb;
             return true;
         }
     }
     return false;
+}
+
+// Threads per block for a pair: 256 when its options ask for it, but 512 for a
+// shape that 8 nodes per thread of 256 hold and two blocks of whole layers do
+// not (a number of layers that is not a multiple of kBlk).
+static int cta_threads(const Geom &g, const gs_solve_opts *o) {
+    if (o->cta_threads != 256) return 512;
+    TileGeom t;
+    int tpt;
+    size_t smem;
+    if (pick_tile(g, t, tpt, smem, o->tile_w, o->tile_h, 256)) return 256;
+    const bool shape = o->tile_w == 4 || o->tile_w == 8 || o->tile_w == 16 || o->tile_w == 32;
+    const size_t fb = shape && o->tile_h > 0 ? field_bytes(g, o->tile_w, o->tile_h, 256) : 0;
+    return fb && fb <= 180 * 1024 ? 512 : 256;
 }
 
 // Per-tile flags are sized for the most tiles any allowed shape gives (4 x 1
@@ -1612,12 +1836,12 @@ size_t tiled_work_extra(const Geom &g) {
 
 // Per-pair arguments from the pair's geometry, state and workspace.
 static int setup_args(const Geom &g, const State &s, const Work &w, const gs_solve_opts *o,
-                      SolveArgs &a, int &npt, size_t &smem, int bt) {
+                      SolveArgs &a, int &tpt, size_t &smem, int bt) {
     memset(&a, 0, sizeof(a));
     a.g = g;
     a.s = s;
-    if (!pick_tile(g, a.t, npt, smem, o->tile_w, o->tile_h, bt)) return GS_ERR_INVAL;
-    a.npt = npt;
+    if (!pick_tile(g, a.t, tpt, smem, o->tile_w, o->tile_h, bt)) return GS_ERR_INVAL;
+    a.tpt = tpt;
     // a step's item count travels in 24 bits of the claim word
     if (a.t.T > (int)(kItemMask - 4096)) return GS_ERR_INVAL;
     char *extra = (char *)w.mark + round_up(g.N * sizeof(int32_t), 256);
@@ -1645,10 +1869,9 @@ static void solve_fields(SolveArgs &a, const gs_solve_opts *o) {
 // Cooperative launch of the batch kernel with the whole grid resident.  The
 // launch goes through cudaLaunchKernelEx with the cooperative attribute, so a
 // caller may capture it in a CUDA graph.
-static int launch_batch(const BatchArgs &B, int npt, size_t smem, int total_tiles, int bt,
+static int launch_batch(const BatchArgs &B, int tpt, size_t smem, int total_tiles, int bt,
                         cudaStream_t st) {
-    void (*kern)(const BatchArgs) = bt == 256 ? (npt == 4 ? k_batch<4, 256> : k_batch<8, 256>)
-                                              : (npt == 4 ? k_batch<4, 512> : k_batch<8, 512>);
+    void (*kern)(const BatchArgs) = tpt == 1 ? k_batch<1> : k_batch<2>;
     int dev = 0;
     GS_CUDA_TRY(cudaGetDevice(&dev));
     int sms = 0, coop = 0;
@@ -1677,7 +1900,7 @@ static int launch_batch(const BatchArgs &B, int npt, size_t smem, int total_tile
 // Control words of a batch launch: the abort flag and finished-pair count,
 // then one PairCtl per pair.
 constexpr size_t kBatchCtrlBytes = 256 + kMaxPairs * sizeof(PairCtl);
-static_assert(256 + kBatchCtrlBytes <= kWorkCtrlBytes, "a pair's workspace holds a batch's control");
+static_assert(512 + sizeof(PairCtl) <= kWorkCtrlBytes, "a pair's workspace holds its control words");
 
 // Idle limit of a launch from one pair's options (0: the default); a batch
 // takes the smallest.
@@ -1686,20 +1909,18 @@ static unsigned long long idle_limit_ns(const gs_solve_opts *o) {
                                 : kDefaultIdleLimitNs;
 }
 
-static int run_batch(BatchArgs &B, int npt, size_t smem, int bt, void *ctrl_mem,
+static int run_batch(BatchArgs &B, int tpt, size_t smem, int bt, void *ctrl_mem,
                      cudaStream_t st) {
     B.bar = (Ctrl *)ctrl_mem;
     B.ctl = (PairCtl *)((char *)ctrl_mem + 256);
     int total = 0;
     for (int p = 0; p < B.n; p++) total += B.pair[p].t.T;
     GS_CUDA_TRY(cudaMemsetAsync(ctrl_mem, 0, 256 + (size_t)B.n * sizeof(PairCtl), st));
-    return launch_batch(B, npt, smem, total, bt, st);
+    return launch_batch(B, tpt, smem, total, bt, st);
 }
 
 size_t batch_ctrl_bytes() { return kBatchCtrlBytes; }
 
-// Threads per block a pair's options ask for.
-static int cta_threads(const gs_solve_opts *o) { return o->cta_threads == 256 ? 256 : 512; }
 
 int tiled_solve(const Geom &g, const State &s, const Work &w, const gs_solve_opts *o,
                 int32_t *status, cudaStream_t st) {
@@ -1710,15 +1931,15 @@ int tiled_solve(const Geom &g, const State &s, const Work &w, const gs_solve_opt
     B.n = 1;
     B.extract = 0;
     B.idle_limit_ns = idle_limit_ns(o);
-    int npt;
+    int tpt;
     size_t smem;
-    const int bt = cta_threads(o);
-    int rc = setup_args(g, s, w, o, B.pair[0], npt, smem, bt);
+    const int bt = cta_threads(g, o);
+    int rc = setup_args(g, s, w, o, B.pair[0], tpt, smem, bt);
     if (rc) return rc;
     solve_fields(B.pair[0], o);
     B.pair[0].status = status;
     GS_CUDA_TRY(cudaMemsetAsync(w.ctrl, 0, sizeof(Ctrl), st));
-    return run_batch(B, npt, smem, bt, (char *)w.ctrl + 256, st);
+    return run_batch(B, tpt, smem, bt, (char *)w.ctrl + 256, st);
 }
 
 int tiled_extract(const Geom &g, const State &s, const Work &w, const gs_solve_opts *o,
@@ -1730,10 +1951,10 @@ int tiled_extract(const Geom &g, const State &s, const Work &w, const gs_solve_o
     B.n = 1;
     B.extract = 1;
     B.idle_limit_ns = idle_limit_ns(o);
-    int npt;
+    int tpt;
     size_t smem;
-    const int bt = cta_threads(o);
-    int rc = setup_args(g, s, w, o, B.pair[0], npt, smem, bt);
+    const int bt = cta_threads(g, o);
+    int rc = setup_args(g, s, w, o, B.pair[0], tpt, smem, bt);
     if (rc) return rc;
     SolveArgs &a = B.pair[0];
     a.hgt = w.mark;
@@ -1743,7 +1964,7 @@ int tiled_extract(const Geom &g, const State &s, const Work &w, const gs_solve_o
     a.labels = labels;
     a.flow = flow;
     a.status = status;
-    return run_batch(B, npt, smem, bt, (char *)w.ctrl + 256, st);
+    return run_batch(B, tpt, smem, bt, (char *)w.ctrl + 256, st);
 }
 
 }  // namespace gs
@@ -1752,14 +1973,14 @@ extern "C" int gs_tile_info(const gs_params *p, const gs_solve_opts *o, int32_t 
     gs::Geom g;
     if (gs::make_geom(p, &g) != GS_OK || !o || !out) return GS_ERR_INVAL;
     gs::TileGeom t;
-    int npt;
-    size_t smem;
-    if (!gs::pick_tile(g, t, npt, smem, o->tile_w, o->tile_h, gs::cta_threads(o)))
+    int tpt;
+    size_t smem, fields;
+    if (!gs::pick_tile(g, t, tpt, smem, o->tile_w, o->tile_h, gs::cta_threads(g, o), &fields))
         return GS_ERR_INVAL;
     out[0] = t.TW;
     out[1] = t.TH;
     out[2] = t.T;
-    out[3] = (int32_t)smem;
+    out[3] = (int32_t)fields;
     return GS_OK;
 }
 
@@ -1784,12 +2005,15 @@ extern "C" int gs_solve_batched(const gs_pair_desc *descs, int32_t n, void *batc
     B.extract = 0;
     E.extract = 1;
     B.idle_limit_ns = kDefaultIdleLimitNs;
-    int npt_max = 4;
+    int tpt_max = 1;
     size_t smem_max = 0;
     // one block size for the launch: 256 threads only when every pair asks
     int bt = 256;
-    for (int i = 0; i < n; i++)
-        if (cta_threads(&descs[i].o) != 256) bt = 512;
+    for (int i = 0; i < n; i++) {
+        Geom g;
+        if (make_geom(&descs[i].p, &g) != GS_OK) return GS_ERR_INVAL;
+        if (cta_threads(g, &descs[i].o) != 256) bt = 512;
+    }
     for (int i = 0; i < n; i++) {
         const gs_pair_desc &d = descs[i];
         Geom g;
@@ -1802,9 +2026,9 @@ extern "C" int gs_solve_batched(const gs_pair_desc *descs, int32_t n, void *batc
         B.idle_limit_ns = std::min(B.idle_limit_ns, idle_limit_ns(&d.o));
         const State s = state_view(d.graph, g);
         const Work w = work_view(d.workspace, g);
-        int npt;
+        int tpt;
         size_t smem;
-        if (setup_args(g, s, w, &d.o, B.pair[i], npt, smem, bt) != GS_OK) return GS_ERR_INVAL;
+        if (setup_args(g, s, w, &d.o, B.pair[i], tpt, smem, bt) != GS_OK) return GS_ERR_INVAL;
         solve_fields(B.pair[i], &d.o);
         B.pair[i].status = d.status;
         E.pair[i] = B.pair[i];
@@ -1815,7 +2039,7 @@ extern "C" int gs_solve_batched(const gs_pair_desc *descs, int32_t n, void *batc
         x.max_iters = 1;
         x.labels = d.labels;
         x.flow = d.flow;
-        npt_max = std::max(npt_max, npt);
+        tpt_max = std::max(tpt_max, tpt);
         smem_max = std::max(smem_max, smem);
     }
     // per pair: data term and graph (small launches), then one launch for all
@@ -1829,7 +2053,7 @@ extern "C" int gs_solve_batched(const gs_pair_desc *descs, int32_t n, void *batc
         GS_CUDA_TRY(cudaMemsetAsync(B.pair[i].ctrl, 0, sizeof(Ctrl), st));
     }
     E.idle_limit_ns = B.idle_limit_ns;
-    int rc = run_batch(B, npt_max, smem_max, bt, batch_ws, st);
+    int rc = run_batch(B, tpt_max, smem_max, bt, batch_ws, st);
     if (rc) return rc;
-    return run_batch(E, npt_max, smem_max, bt, batch_ws, st);
+    return run_batch(E, tpt_max, smem_max, bt, batch_ws, st);
 }

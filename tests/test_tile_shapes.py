@@ -1,0 +1,59 @@
+"""Tile shapes of the persistent solver at their edges: blocks of four chain
+layers with 1 to 4 layers left in the last one, one or two blocks per thread,
+tile widths with code of their own (8, 16) and without (4, 32), rows that do
+not fill a warp, tiles that the grid cuts off."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("bt,tile,D,fits", [
+    (256, (32, 3), 22, True),     # two blocks per thread of 512, not of 256
+    (256, (8, 3), 86, True),
+    (512, (32, 8), 16, True),     # 256 sites x 15 layers: nine fields of exactly 180 KB
+    (512, (32, 8), 17, False),
+    (512, (4, 1), 280, True),     # long chains, the narrowest tile
+    (256, (8, 9), 4, False),
+])
+def test_shapes_accepted(bt, tile, D, fits):
+    from paper_1803_01516_gb300 import build
+    build.build()
+    from paper_1803_01516_gb300 import gazecut as gc
+    p = gc.Params(w=2 * (D - 1) + 64, h=40, D=D, tau=30, lam=3)
+    o = gc.SolveOpts(cta_threads=bt, tile_w=tile[0], tile_h=tile[1])
+    if fits:
+        info = gc.gs_tile_info(p, o)
+        assert (info["tile_w"], info["tile_h"]) == tile
+        assert info["smem_bytes"] <= 180 * 1024
+    else:
+        with pytest.raises(RuntimeError):
+            gc.gs_tile_info(p, o)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D", [2, 4, 5, 6, 7, 8, 18])
+@pytest.mark.parametrize("tile,bt", [((8, 8), 256), ((8, 8), 512), ((16, 8), 512), ((16, 8), 256),
+                                     ((32, 8), 512), ((32, 3), 256), ((4, 8), 256), ((4, 1), 512),
+                                     ((8, 3), 256), ((16, 5), 512)])
+def test_tile_edges_exact(D, tile, bt):
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1803_01516_gb300 import gazecut as gc
+    h, ng = 19, 43                                   # no tile divides either
+    rng = np.random.default_rng(100 * D + tile[0] + tile[1])
+    C = rng.integers(0, 31, size=(h, ng, D)).astype(np.int32)
+    p = gc.Params(w=ng + 2 * (D - 1), h=h, D=D, tau=0, lam=4, inhibit=37)
+    o = gc.SolveOpts(cta_threads=bt, tile_w=tile[0], tile_h=tile[1])
+    try:
+        gc.gs_tile_info(p, o)
+    except RuntimeError:
+        pytest.skip("the shape does not fit this depth range")
+    ref = oracle.solve(C, 4, 37, 1)
+    for direction in (1, 2):
+        p.direction = direction
+        X, flow, status = gc.solve_costs(torch.from_numpy(C).cuda(), p, o)
+        assert int(status.item()) == gc.GS_OK and int(flow.item()) == ref["flow"]
+        assert np.array_equal(X.cpu().numpy(), ref["labels"])
