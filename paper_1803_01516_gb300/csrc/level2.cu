@@ -9,8 +9,11 @@
 // for n labels), the row cost holds the sites' data and border terms and the
 // pairs inside the row, and the pairs between consecutive rows -- a sum over
 // the columns -- are applied one column at a time (a min-plus transform of one
-// label digit), so moving from row to row costs bw * n^(bw+1) operations
-// instead of n^(2 bw).  Forward and backward passes give every row state's
+// label digit).  The transform is linear in n: h~ is the min-plus convolution
+// of lambda |d| on |d| <= 1 (infinite beyond) with (lambda + inhibit) |d|, so a
+// line of n labels takes a three-point minimum and one running minimum each
+// way.  Moving from row to row costs 2 bw n^bw steps, instead of n^(2 bw) for
+// all pairs of states or bw n^(bw+1) for all pairs of labels.  Forward and backward passes give every row state's
 // min-marginal; the smallest label a site takes in any minimiser, read from
 // the states whose min-marginal equals the minimum, is the site's label in the
 // component-wise smallest minimiser (the minimisers of this convex-prior
@@ -37,33 +40,52 @@ struct L2Args {
     long long lam, h2h, h2v;
 };
 
-// Min-plus transform of label digit c of every row state: out(s) = min over d
-// of in(s with digit c = d) + h~_v(d - digit_c(s)).
-__device__ __forceinline__ void col_transform(const long long *in, long long *out, int S, int n,
-                                              int pw, long long lam, long long inh, int lane) {
-    for (int s = lane; s < S; s += 32) {
-        const int dc = (s / pw) % n;
-        const int base = s - dc * pw;
-        long long best = kL2Inf * 64;
-        for (int d = 0; d < n; d++) best = min(best, in[base + d * pw] + htil(d - dc, lam, inh));
-        out[s] = best;
+// Min-plus transform of one label digit of every row state (states whose other
+// digits agree lie pw apart, n of them: a line): out = min over d of in(d) +
+// h~_v(d - digit), in place when in == out.  One line a lane: the lane holds
+// the line's previous inputs, so it may overwrite them.
+__device__ __forceinline__ void col_transform(const long long *in, long long *out, int lines, int n,
+                                              unsigned rn, int pw, bool top, long long lam,
+                                              long long inh, int lane) {
+    for (int q = lane; q < lines; q += 32) {
+        // the line's first state: q with a digit 0 put in at pw
+        const int hi = pw == 1 ? q : top ? 0 : n == 1 ? q : (int)__umulhi((unsigned)q, rn);
+        const int base = pw == 1 ? q * n : q - hi * pw + hi * pw * n;
+        long long cur = in[base], prev = kL2Inf * 64, run = kL2Inf * 64;
+        for (int d = 0; d < n; d++) {
+            const long long next = d + 1 < n ? in[base + (d + 1) * pw] : kL2Inf * 64;
+            const long long m = min(cur, min(prev, next) + lam);
+            run = min(m, run + lam + inh);
+            out[base + d * pw] = run;
+            prev = cur;
+            cur = next;
+        }
+        for (int d = n - 2; d >= 0; d--) {
+            run = min(out[base + d * pw], run + lam + inh);
+            out[base + d * pw] = run;
+        }
     }
     __syncwarp();
 }
 
+// One warp per block.  Bound by the latency of the lines' running minima and
+// by how many warps hide it: 4 S + 96 words of 8 bytes a warp (S row states, 729
+// for 3 x 3 sites and 9 labels) leave room for eight warps per SM.  384x288x16
+// at b = 3, four half-passes over 11,000 blocks: 4.37 ms with the transform over
+// all pairs of labels and its own two buffers (four warps per SM), 0.90 ms now.
 __global__ void __launch_bounds__(32 * kL2Warps) k_block_descent(const L2Args a) {
     extern __shared__ long long l2sm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S_cap = a.scap;
-    long long *F = l2sm + (size_t)warp * (6 * S_cap + 96);   // F[3][S_cap]
+    long long *F = l2sm + (size_t)warp * (4 * S_cap + 96);   // F[3][S_cap]
     long long *Bk = F + 3 * S_cap;
-    long long *A = Bk + S_cap;
-    long long *Bb = A + S_cap;
-    long long *U = Bb + S_cap;                                 // [bh][bw][n], at most 96
-    const int nblocks = a.nbx * a.nby;
+    long long *U = Bk + S_cap;                                 // [bh][bw][n], at most 96
+    // the colour's blocks: n_even in an even row of blocks, nbx in two rows
+    const int n_even = (a.nbx + 1 - a.colour) / 2;
+    const int nblocks = a.nby / 2 * a.nbx + (a.nby & 1) * n_even;
     for (int k = blockIdx.x * kL2Warps + warp; k < nblocks; k += gridDim.x * kL2Warps) {
-        const int bx = k % a.nbx, by = k / a.nbx;
-        if (((bx + by) & 1) != a.colour) continue;
+        const int pair = k / a.nbx, rest = k - pair * a.nbx, odd = rest >= n_even;
+        const int by = 2 * pair + odd, bx = 2 * (rest - odd * n_even) + ((by + a.colour) & 1);
         const int y0 = by * a.b, W0 = bx * a.b;
         const int bh = min(a.b, a.h - y0), bw = min(a.b, a.ng - W0);
         // the block's label range: the union of its sites' bounds
@@ -90,6 +112,7 @@ __global__ void __launch_bounds__(32 * kL2Warps) k_block_descent(const L2Args a)
             if (lane == 0) atomicCAS(a.status, GS_OK, GS_ERR_INVAL);
             continue;
         }
+        const unsigned rn = n > 1 ? (unsigned)((0x100000000ull + n - 1) / n) : 0u;   // for s / n
         // unary terms: data term inside the site's bounds, plus the pairs to
         // sites outside the block against their current labels
         for (int t = lane; t < bh * bw * n; t += 32) {
@@ -112,29 +135,31 @@ __global__ void __launch_bounds__(32 * kL2Warps) k_block_descent(const L2Args a)
         // row cost of state s in row r (data, border terms, pairs inside the row)
         auto row_cost = [&](int r, int s) {
             long long acc = 0;
-            int prev = -1;
+            int prev = 0;
             for (int c = 0; c < bw; c++) {
-                const int d = s % n;
-                s /= n;
+                const int q = n > 1 ? (int)__umulhi((unsigned)s, rn) : s;
+                const int d = s - q * n;
+                s = q;
                 acc += U[(r * bw + c) * n + d];
                 if (c > 0) acc += htil(prev - d, a.lam, a.h2h);
                 prev = d;
             }
             return acc;
         };
+        // min-plus step to the next row, digit by digit, from src into dst
+        auto row_step = [&](const long long *src, long long *dst) {
+            int pw = 1;
+            for (int c = 0; c < bw; c++, pw *= n)
+                col_transform(c == 0 ? src : dst, dst, S / n, n, rn, pw, c == bw - 1, a.lam, a.h2v,
+                              lane);
+        };
         // forward
         for (int s = lane; s < S; s += 32) F[s] = row_cost(0, s);
         __syncwarp();
         for (int r = 1; r < bh; r++) {
-            const long long *src = F + (r - 1) * S_cap;
-            long long *bufs[2] = {A, Bb};
-            int pw = 1;
-            for (int c = 0; c < bw; c++, pw *= n) {
-                col_transform(c == 0 ? src : bufs[(c - 1) & 1], bufs[c & 1], S, n, pw, a.lam, a.h2v,
-                              lane);
-            }
-            const long long *G = bufs[(bw - 1) & 1];
-            for (int s = lane; s < S; s += 32) F[r * S_cap + s] = row_cost(r, s) + G[s];
+            long long *Fr = F + r * S_cap;
+            row_step(F + (r - 1) * S_cap, Fr);
+            for (int s = lane; s < S; s += 32) Fr[s] += row_cost(r, s);
             __syncwarp();
         }
         // minimum energy of the block problem
@@ -147,31 +172,28 @@ __global__ void __launch_bounds__(32 * kL2Warps) k_block_descent(const L2Args a)
         for (int r = bh - 1; r >= 0; r--) {
             if (r < bh - 1) {
                 // Bk_r(s) = min over s' of V(s, s') + R_(r+1)(s') + Bk_(r+1)(s')
-                for (int s = lane; s < S; s += 32) A[s] = row_cost(r + 1, s) + Bk[s];
+                for (int s = lane; s < S; s += 32) Bk[s] += row_cost(r + 1, s);
                 __syncwarp();
-                long long *bufs[2] = {Bb, A};
-                int pw = 1;
-                for (int c = 0; c < bw; c++, pw *= n) {
-                    col_transform(c == 0 ? A : bufs[(c - 1) & 1], bufs[c & 1], S, n, pw, a.lam,
-                                  a.h2v, lane);
-                }
-                const long long *G = bufs[(bw - 1) & 1];
-                for (int s = lane; s < S; s += 32) Bk[s] = G[s];
-                __syncwarp();
+                row_step(Bk, Bk);
             }
-            for (int c = 0; c < bw; c++) {
-                int best = n;
-                int pw = 1;
-                for (int q = 0; q < c; q++) pw *= n;
-                for (int s = lane; s < S; s += 32)
-                    if (F[r * S_cap + s] + Bk[s] == Emin) best = min(best, (s / pw) % n);
-                for (int o = 16; o > 0; o >>= 1)
-                    best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
-                if (lane == 0) {
-                    const int64_t v = (int64_t)(y0 + r) * a.ng + W0 + c;
-                    if (best < n) a.labels[v] = LO + best;
-                    else atomicCAS(a.status, GS_OK, GS_ERR_LABELS);
+            int best[3] = {n, n, n};             // bw <= 3
+            for (int s = lane; s < S; s += 32) {
+                if (F[r * S_cap + s] + Bk[s] != Emin) continue;
+                int rest = s;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const int q = n > 1 ? (int)__umulhi((unsigned)rest, rn) : rest;
+                    best[c] = min(best[c], rest - q * n);
+                    rest = q;
                 }
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++) best[c] = __reduce_min_sync(0xffffffffu, best[c]);
+            if (lane < bw) {
+                const int d = lane == 0 ? best[0] : lane == 1 ? best[1] : best[2];
+                const int64_t v = (int64_t)(y0 + r) * a.ng + W0 + lane;
+                if (d < n) a.labels[v] = LO + d;
+                else atomicCAS(a.status, GS_OK, GS_ERR_LABELS);
             }
             __syncwarp();
         }
@@ -261,7 +283,7 @@ extern "C" int gs_block_descent(const int32_t *cost, const gs_params *p, int32_t
     a.lam = g.lam;
     a.h2h = g.h2h;
     a.h2v = g.h2v;
-    const size_t smem = (size_t)kL2Warps * (6 * a.scap + 96) * sizeof(long long);
+    const size_t smem = (size_t)kL2Warps * (4 * a.scap + 96) * sizeof(long long);
     GS_CUDA_TRY(cudaFuncSetAttribute(k_block_descent, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));
     const int64_t half = ((int64_t)a.nbx * a.nby + 1) / 2;
