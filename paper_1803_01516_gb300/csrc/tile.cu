@@ -115,6 +115,9 @@ __device__ __forceinline__ unsigned long long atom_add_relaxed(unsigned long lon
     asm volatile("atom.relaxed.gpu.global.add.u64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(v) : "memory");
     return r;
 }
+__device__ __forceinline__ void red_add_release(unsigned *p, unsigned v) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ unsigned long long atom_exch_release(unsigned long long *p,
                                                               unsigned long long v) {
     unsigned long long r;
@@ -210,13 +213,14 @@ __device__ __forceinline__ int32_t atom_add_nz(unsigned a, int32_t v) {
                  "  @q atom.shared.add.s32 %0, [%1], %2; }" : "=&r"(r) : "r"(a), "r"(v));
     return r;
 }
-// Add w to the word at a, and v to the one at b, each if it is not 0; returns what b held
-// before (0 if it was left alone).
-__device__ __forceinline__ int32_t push_words(unsigned a, int32_t w, unsigned b, int32_t v) {
+// Store w at a where p is not 0, and add v to the word at b if it is not 0;
+// returns what b held before (0 if it was left alone).
+__device__ __forceinline__ int32_t push_words(unsigned a, int32_t w, int32_t p, unsigned b,
+                                              int32_t v) {
     int32_t r;
-    asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %2, 0; setp.ne.s32 q, %4, 0; mov.s32 %0, 0;"
-                 "  @p red.shared.add.s32 [%1], %2; @q atom.shared.add.s32 %0, [%3], %4; }"
-                 : "=&r"(r) : "r"(a), "r"(w), "r"(b), "r"(v));
+    asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %3, 0; setp.ne.s32 q, %5, 0; mov.s32 %0, 0;"
+                 "  @p st.volatile.shared.s32 [%1], %2; @q atom.shared.add.s32 %0, [%4], %5; }"
+                 : "=&r"(r) : "r"(a), "r"(w), "r"(p), "r"(b), "r"(v));
     return r;
 }
 // Add v to a global word unless it is 0, and store v where p holds: no branch.
@@ -576,8 +580,9 @@ __shared__ unsigned s_sides;
 // heights reset (0 on nodes with sink capacity left, else infinity), local
 // relaxation with an unknown (infinite) halo.  Returns the tile's active
 // count (positive excess and a finite height).
-template <int TPT, int TWC>
-__device__ __forceinline__ int relabel_init_tile(const SolveArgs &a, int32_t *sm, int tile) {
+template <int TPT, int TWC, class Halfway>
+__device__ __forceinline__ int relabel_init_tile(const SolveArgs &a, int32_t *sm, int tile,
+                                                 Halfway halfway) {
     const Geom &g = a.g;
     const TileGeom &t = a.t;
     const State &s = a.s;
@@ -645,6 +650,7 @@ __device__ __forceinline__ int relabel_init_tile(const SolveArgs &a, int32_t *sm
     }
     halo_rest<TWC>(a, sm, l, o, true, nullptr);
     __syncthreads();
+    halfway();
 #pragma unroll
     for (int u = 0; u < TPT; u++) {
 #pragma unroll
@@ -714,10 +720,10 @@ __device__ __forceinline__ int side_tile(const TileGeom &t, const TileOrigin &o,
 // memory (own and halo); relax, write back what changed, mark the neighbour
 // tiles whose halo changed, and return the change of the tile's active count
 // (the marks are warp 0's and come after the visit's last block barrier).
-template <int TPT, int TWC>
+template <int TPT, int TWC, class Halfway>
 __device__ __forceinline__ int relabel_pass_tile(const SolveArgs &a, int32_t *sm, int tile, int &changed,
                                  int32_t *dirty_next, int32_t *list_next, int32_t *count_next,
-                                 const unsigned *done_ctr, unsigned items) {
+                                 const unsigned *done_ctr, unsigned items, Halfway halfway) {
     const Geom &g = a.g;
     const TileGeom &t = a.t;
     const Lay<TWC> l(t);
@@ -761,6 +767,7 @@ __device__ __forceinline__ int relabel_pass_tile(const SolveArgs &a, int32_t *sm
             if (cell[u] && k < nl[u]) sm[abs(cell[u]) + l.at(F_HT, k)] = h0[u][k];
     halo_rest<TWC>(a, sm, l, o, false, a.hgt);
     __syncthreads();
+    halfway();
     bool cut = false;
     const bool ch = relax_tile<TPT, TWC>(a, sm, cell, nl, mk, 1 << 30, done_ctr, items, &cut);
     int act = 0;
@@ -874,10 +881,10 @@ __device__ __forceinline__ void discharge(const Lay<TWC> &l, unsigned base, unsi
     c = base + 4 * c;
     int32_t e = lds(c + 4 * l.at(F_EX));
     const int32_t hu = lds(c + 4 * l.at(F_HT));
-    int32_t r[4], hv[4], x[4];
+    int32_t w[4], hv[4], x[4];
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-        r[j] = lds(c + st[j].x);
+        w[j] = lds(c + st[j].x);
         hv[j] = lds(c + st[j].y + 4 * l.at(F_HT));
     }
     if (i >= n) e = 0;
@@ -885,10 +892,10 @@ __device__ __forceinline__ void discharge(const Lay<TWC> &l, unsigned base, unsi
     unsigned sum = 0;
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-        r[j] = (int32_t)((unsigned)st[j].z + (unsigned)st[j].w * (unsigned)r[j]);
+        const int32_t r = (int32_t)((unsigned)st[j].z + (unsigned)st[j].w * (unsigned)w[j]);
         // (a head that does not exist has an infinite height)
-        x[j] = r[j] > 0 && hv[j] < hu ? min(r[j], e) : 0;
-        hm = min(hm, r[j] > 0 && hv[j] >= hu ? hv[j] : kInfH);
+        x[j] = r > 0 && hv[j] < hu ? min(r, e) : 0;
+        hm = min(hm, r > 0 && hv[j] >= hu ? hv[j] : kInfH);
         sum = min(sum + (unsigned)x[j], (unsigned)e);
     }
 #pragma unroll
@@ -907,7 +914,10 @@ __device__ __forceinline__ void discharge(const Lay<TWC> &l, unsigned base, unsi
         x[j] = min(x[j], left);
         left -= x[j];
         ea[j] = c + st[j].y + 4 * l.at(F_EX);
-        old[j] = push_words(c + st[j].x, st[j].w > 0 ? -x[j] : x[j], ea[j],
+        // (the arc's word needs no atomic: in one iteration only one of its ends
+        // can push along it -- each would have to lie above the other, and
+        // heights only rise)
+        old[j] = push_words(c + st[j].x, st[j].w > 0 ? w[j] - x[j] : w[j] + x[j], x[j], ea[j],
                             j == 2 && own ? -tot : x[j]);
     }
     // lane 3: every admissible slot is saturated: relabel over the others
@@ -932,10 +942,10 @@ __device__ __forceinline__ void discharge(const Lay<TWC> &l, unsigned base, unsi
 
 // Up to `iters` push/relabel iterations of one tile in shared memory.  (The
 // queueing at the end is warp 0's and comes after the visit's last barrier.)
-template <int TPT, int TWC>
+template <int TPT, int TWC, class Halfway>
 __device__ __forceinline__ void sweep_tile(const SolveArgs &a, int32_t *sm, int tile, int round, int iters,
                            int &overflow, int32_t *list_next, int32_t *count_next,
-                           const unsigned *done_ctr, unsigned items) {
+                           const unsigned *done_ctr, unsigned items, Halfway halfway) {
     const Geom &g = a.g;
     const TileGeom &t = a.t;
     const State &s = a.s;
@@ -1005,6 +1015,7 @@ __device__ __forceinline__ void sweep_tile(const SolveArgs &a, int32_t *sm, int 
     }
     halo_rest<TWC>(a, sm, l, o, true, s.ht);
     __syncthreads();
+    halfway();
     // the first list
     const unsigned base = (unsigned)__cvta_generic_to_shared(sm);
     const unsigned lists = base + 4 * (t.words + t.nblk + 2), nowhere = lists + 4 * t.TN;
@@ -1356,31 +1367,53 @@ __device__ void advance(PairState &st, const SolveArgs &a, const long long v[4],
     }
 }
 
-// Labels of one tile's sites and the tile's remaining sink capacity.
-__device__ long long labels_tile(const SolveArgs &a, int tile, const int32_t *hsrc, int &bad) {
+// Labels of one tile's sites and the tile's remaining sink capacity.  A thread
+// counts the source-side nodes of its blocks of layers; the source side of a
+// chain must be a prefix, so a source-side node lies above another or is the
+// first.  (One thread per site walked the whole chain with the other threads
+// idle: 1.85 ms for 514x480 sites of 63 layers.)
+__device__ long long labels_tile(const SolveArgs &a, int32_t *sm, int tile, const int32_t *hsrc,
+                                 int &bad) {
     const Geom &g = a.g;
     const TileGeom &t = a.t;
     const TileOrigin o = tile_origin(t, tile);
+    int32_t *count = sm + t.words + t.nblk + 2;      // [S], where sweeps keep their lists
     unsigned long long deficit = 0;
     int b = 0;
     const int dir = eff_dir(a);
     const bool rev = ld(&a.s.hdr->rev) != 0;
-    for (int sidx = threadIdx.x; sidx < t.TW * t.TH; sidx += blockDim.x) {
-        const int wl = sidx % t.TW, yl = sidx / t.TW;
-        const int W = o.W0 + wl, y = o.y0 + yl;
-        if (W >= g.ng || y >= g.h) continue;
-        int64_t i = (int64_t)y * g.SY + W;
-        int lab = 0, prev = 1;
-        for (int j = 0; j < g.K; j++, i += g.P) {
-            const int32_t h = ld(&hsrc[i]);
-            const int in = dir == 1 ? (h < kInfH) : (h >= kInfH);
-            b |= in && !prev;
-            lab += in;
-            prev = in;
-            const int32_t e = ld(&a.s.ex[i]);
-            if (e < 0) deficit += (unsigned long long)(-(int64_t)e);
+    for (int site = threadIdx.x; site < t.S; site += blockDim.x) count[site] = 0;
+    __syncthreads();
+    for (int u = 0; u < a.tpt; u++) {
+        const Own w = own_block<0>(g, t, u);
+        const int W = o.W0 + w.wl, y = o.y0 + w.yl;
+        if (!w.n || W >= g.ng || y >= g.h) continue;
+        const int64_t i = ((int64_t)y * g.K + w.j0) * g.P + W;
+        int32_t h[kBlk + 1], e[kBlk];
+#pragma unroll
+        for (int k = 0; k <= kBlk; k++)              // h[0]: the layer below the block
+            h[k] = k <= w.n && w.j0 + k > 0 ? ld(&hsrc[i + (int64_t)(k - 1) * g.P]) : 0;
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) e[k] = k < w.n ? ld(&a.s.ex[i + (int64_t)k * g.P]) : 0;
+        auto in = [&](int32_t v) { return dir == 1 ? v < kInfH : v >= kInfH; };
+        bool prev = w.j0 == 0 || in(h[0]);
+        int n = 0;
+#pragma unroll
+        for (int k = 0; k < kBlk; k++) {
+            if (k >= w.n) break;
+            const bool now = in(h[k + 1]);
+            b |= now && !prev;
+            n += now;
+            prev = now;
+            if (e[k] < 0) deficit += (unsigned long long)(-(int64_t)e[k]);
         }
-        a.labels[(int64_t)y * g.ng + W] = rev ? g.D - 1 - lab : lab;
+        if (n) atomicAdd(&count[w.yl * t.TW + w.wl], n);
+    }
+    __syncthreads();
+    for (int site = threadIdx.x; site < t.S; site += blockDim.x) {
+        const int yl = site / t.TW, W = o.W0 + site - yl * t.TW, y = o.y0 + yl;
+        if (W < g.ng && y < g.h)
+            a.labels[(int64_t)y * g.ng + W] = rev ? g.D - 1 - count[site] : count[site];
     }
     bad = __syncthreads_or(b);
     return block_sum((long long)deficit);
@@ -1491,6 +1524,28 @@ struct Item {
     unsigned items, idx;    // items of the step, this one's number
 };
 
+// The block's next item of the same step, claimed while it works on this one
+// (thread 0): the claim's result, then the tile it names.  Only while the step
+// has two items or more left for every block, so that its end stays shared out.
+struct Ahead {
+    unsigned long long w;
+    int32_t tile, count;    // queued tile (or the item's number); its active nodes
+    int abort;
+    bool has;
+};
+
+// Halfway through a visit (thread 0): look up the item claimed ahead.
+__device__ __forceinline__ void look_ahead(const BatchArgs &B, const SolveArgs &a, const Item &it,
+                                           bool queued, Ahead &ah) {
+    if (threadIdx.x != 0 || !ah.has) return;
+    const unsigned idx = (unsigned)(ah.w & kItemMask);
+    ah.has = idx < it.items;
+    if (!ah.has) return;
+    ah.tile = queued ? ld(&a.tile_list[it.slot * a.t.T + idx]) : (int)idx;
+    ah.count = ld(&a.tile_cnt[idx]);
+    ah.abort = *(volatile int32_t *)&B.bar->abort;
+}
+
 // Sums of a completed item (active nodes or worked tiles, changes, visits, overflow).
 struct ItemSums {
     long long a, b, c;
@@ -1503,11 +1558,33 @@ struct ItemSums {
 // The atomic that claims the next item of the same step goes out before the
 // one that counts the completed item, so the two round trips overlap; the
 // words a claimed item needs are loaded by one lane each.
+// With an item claimed ahead there is nothing to wait for: this one cannot be
+// the step's last, so it is counted without looking at the count, and the
+// pair's state is the same.
 __device__ __forceinline__ void next_item(const BatchArgs &B, Item &it, const ItemSums &v0,
-                                          PairState &s_st) {
+                                          const Ahead &ah, PairState &s_st) {
     const int lane = threadIdx.x & 31;
     ItemSums v = v0;
     bool finish = it.tile >= 0;
+    if (__shfl_sync(0xffffffffu, (int)ah.has, 0)) {
+        if (lane == 0) {
+            PairCtl *c = B.ctl + it.p;
+            long long *rp = c->red[it.slot];
+            if (v.a) atomicAdd((unsigned long long *)&rp[0], (unsigned long long)v.a);
+            if (v.b) atomicAdd((unsigned long long *)&rp[1], (unsigned long long)v.b);
+            if (v.c) atomicAdd((unsigned long long *)&rp[2], (unsigned long long)v.c);
+            if (v.ovf) atomicAdd((unsigned long long *)&rp[3], 1ull);
+            red_add_release(&c->done, 1u);
+        }
+        it.idx = (unsigned)(__shfl_sync(0xffffffffu, ah.w, 0) & kItemMask);
+        it.tile = __shfl_sync(0xffffffffu, ah.tile, 0);
+        if (__shfl_sync(0xffffffffu, ah.abort, 0)) it.tile = -1;
+        if (it.tile < 0 || queued(s_st) || s_st.phase != PH_SWEEP ||
+            __shfl_sync(0xffffffffu, ah.count, 0) > 0)
+            return;
+        v.a = v.b = v.c = 0;             // nothing to sweep in that tile
+        v.ovf = 0;
+    }
     for (;;) {
         unsigned long long w = 0;
         bool got = false;
@@ -1594,11 +1671,16 @@ __device__ __forceinline__ void next_item(const BatchArgs &B, Item &it, const It
 struct Visit {
     int tile, next, T;
     unsigned items;
+    const BatchArgs &B;
+    const Item &it;
 };
 
 template <int TPT, int TWC>
 __device__ __forceinline__ void visit_tile(const SolveArgs &a, PairCtl *c, const PairState &st,
-                                           const Visit &v, int32_t *sm, ItemSums &sums) {
+                                           const Visit &v, int32_t *sm, ItemSums &sums,
+                                           Ahead &ah) {
+    // between a visit's staging and its work, when the claim ahead is back
+    auto halfway = [&]() { look_ahead(v.B, a, v.it, queued(st), ah); };
     int32_t *list_next = a.tile_list + v.next * v.T;
     int32_t *count_next = &c->qcount[v.next];
     const int tile = v.tile;
@@ -1609,7 +1691,7 @@ __device__ __forceinline__ void visit_tile(const SolveArgs &a, PairCtl *c, const
             __stcg(&a.tile_act[tile], 0);
             __stcg(&a.tile_act[v.T + tile], 0);
         }
-        sums.a = relabel_init_tile<TPT, TWC>(a, sm, tile);
+        sums.a = relabel_init_tile<TPT, TWC>(a, sm, tile, halfway);
         sums.c = 1;
     } else if (st.phase == PH_PASS) {
         const int pass = st.pass;
@@ -1618,7 +1700,7 @@ __device__ __forceinline__ void visit_tile(const SolveArgs &a, PairCtl *c, const
         if (pass > 1 && threadIdx.x == 0) __stcg(&dcur[tile], 0);
         int ch = 0;
         sums.a = relabel_pass_tile<TPT, TWC>(a, sm, tile, ch, dnext, list_next, count_next, &c->done,
-                                             v.items);
+                                             v.items, halfway);
         sums.b = ch;
         sums.c = 1;
     } else {   // PH_SWEEP
@@ -1627,7 +1709,7 @@ __device__ __forceinline__ void visit_tile(const SolveArgs &a, PairCtl *c, const
         const int iters = st.tail ? a.tail_iters : a.local_iters;
         const unsigned *done_ctr = a.mode == GS_MODE_FIXED_SWEEPS ? nullptr : &c->done;
         sweep_tile<TPT, TWC>(a, sm, tile, cur, iters, sums.ovf, list_next, count_next, done_ctr,
-                             v.items);
+                             v.items, halfway);
         sums.a = 1;
     }
 }
@@ -1674,9 +1756,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_batch(const __grid_constant
     }
     Item it = {0, -1, 0, 0, 0};
     ItemSums sums = {0, 0, 0, 0};
+    Ahead ah = {0, 0, 0, 0, false};
     for (;;) {
         if (threadIdx.x < 32) {
-            next_item(B, it, sums, s_st);
+            next_item(B, it, sums, ah, s_st);
             if (threadIdx.x == 0) s_item = it;
         }
         __syncthreads();
@@ -1690,25 +1773,27 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_batch(const __grid_constant
             __syncthreads();
         }
         sums = {0, 0, 0, 0};
+        ah.has = threadIdx.x == 0 && it.idx + 2 * gridDim.x < it.items;
+        if (ah.has) ah.w = atom_add_relaxed(&c->claim, 1ull);
         // (a visit has a block barrier after its last look at s_item and s_st,
         // and ends with warp 0's queueing)
         if (s_st.phase != PH_LABELS) {
             // the visit's code for this tile width, and a pair whose tiles
             // need one block per thread runs that code also when the launch is
             // sized for two
-            const Visit v = {it.tile, (it.slot + 1) % 3, a.t.T, it.items};
+            const Visit v = {it.tile, (it.slot + 1) % 3, a.t.T, it.items, B, it};
             if (TPT == 2 && a.tpt == 1) {
-                if (a.t.TW == 8) visit_tile<1, 8>(a, c, s_st, v, smem, sums);
-                else if (a.t.TW == 16) visit_tile<1, 16>(a, c, s_st, v, smem, sums);
-                else visit_tile<1, 0>(a, c, s_st, v, smem, sums);
+                if (a.t.TW == 8) visit_tile<1, 8>(a, c, s_st, v, smem, sums, ah);
+                else if (a.t.TW == 16) visit_tile<1, 16>(a, c, s_st, v, smem, sums, ah);
+                else visit_tile<1, 0>(a, c, s_st, v, smem, sums, ah);
             } else {
-                if (a.t.TW == 8) visit_tile<TPT, 8>(a, c, s_st, v, smem, sums);
-                else if (a.t.TW == 16) visit_tile<TPT, 16>(a, c, s_st, v, smem, sums);
-                else visit_tile<TPT, 0>(a, c, s_st, v, smem, sums);
+                if (a.t.TW == 8) visit_tile<TPT, 8>(a, c, s_st, v, smem, sums, ah);
+                else if (a.t.TW == 16) visit_tile<TPT, 16>(a, c, s_st, v, smem, sums, ah);
+                else visit_tile<TPT, 0>(a, c, s_st, v, smem, sums, ah);
             }
         } else {
             int bad = 0;
-            sums.a = labels_tile(a, it.tile, s_st.ht_labels ? a.s.ht : a.hgt, bad);
+            sums.a = labels_tile(a, smem, it.tile, s_st.ht_labels ? a.s.ht : a.hgt, bad);
             sums.b = bad;
         }
         __syncwarp();
