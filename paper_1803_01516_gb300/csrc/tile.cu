@@ -1793,6 +1793,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_batch(const __grid_constant
             }
         } else {
             int bad = 0;
+            look_ahead(B, a, it, false, ah);
             sums.a = labels_tile(a, smem, it.tile, s_st.ht_labels ? a.s.ht : a.hgt, bad);
             sums.b = bad;
         }
