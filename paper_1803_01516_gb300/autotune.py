@@ -10,9 +10,9 @@ the tests) with CUDA events, the best median over a few runs kept.
 
 The cache lives in $GAZECUT_TUNE_CACHE or ~/.cache/gazecut_gb300/autotune.json;
 buckets missing there fall back to ``tuned_defaults.json`` beside this module
-(a tile shape and block size per bucket, measured on a GB300; the schedule is
-the library's own rule, which beat the schedules tuned per bucket by 10 % over
-21 sizes), then to the library defaults.
+(a block size per bucket, and a tile shape where one beats the library's own,
+measured on a GB300; the schedule is the library's own rule, which beat the
+schedules tuned per bucket by 10 % over 21 sizes), then to the library defaults.
 """
 from __future__ import annotations
 
@@ -27,7 +27,8 @@ from . import synth
 
 SCHEDULES = [(spr, li, rp, tf) for spr in (8, 16, 32, 64) for li in (4, 8, 16) for rp in (4, 8, 16)
              for tf in (2, 4)]       # tf: tail iterations = tf x local iterations
-SHAPES = [(16, 8), (8, 8), (16, 4), (32, 4), (8, 4), (16, 2), (8, 2), (4, 4)]
+SHAPES = [(16, 8), (16, 6), (8, 8), (16, 4), (32, 4), (8, 7), (8, 6), (8, 5), (8, 4), (16, 2),
+          (8, 2), (4, 4)]
 CTA_THREADS = (512, 256)     # one block per SM, or two half-size blocks
 
 

@@ -1858,12 +1858,18 @@ static size_t field_bytes(const Geom &g, int TW, int TH, int bt) {
 static bool pick_tile(const Geom &g, TileGeom &t, int &tpt, size_t &smem, int want_w = 0,
                       int want_h = 0, int bt = kTileThreads, size_t *fields = nullptr) {
     const size_t budgets[2] = {(bt == 256 && !want_w ? 80 : 180) * size_t(1024), 180 * 1024};
-    // more sites first, squarer first among equals: a breadth-first path then
-    // crosses fewer tile borders (measured: 8x8 beats 16x4 at 31 depth layers,
-    // 8x4 beats 16x2 at 47)
-    static const int cand[][2] = {{16, 8}, {8, 8}, {16, 4}, {32, 4}, {8, 4}, {32, 2},
-                                  {16, 2}, {4, 8}, {8, 2},  {4, 4},  {16, 1}, {8, 1},
-                                  {4, 2},  {4, 1}};
+    // More sites first, squarer first among equals: a breadth-first path then
+    // crosses fewer tile borders, and a visit's fixed cost (staging, claims,
+    // write-back: half of it) is spread over more sites.  With the number of
+    // blocks of layers between two powers of two only rows of 5, 6 or 7 sites
+    // fill the threads.  500x300 pairs, 512 threads, ms: 20 depth numbers 8x8
+    // 22.0, 16x6 18.3; 36: 8x4 39.3, 8x7 29.2; 44: 8x4 42.2, 8x5 36.9; 700x400x40:
+    // 8x4 93.8, 8x6 68.4, and 8x8 with two blocks per thread 79.5 (its visits
+    // spill); 32: 8x8 24.7, 8x7 26.1.  16x5 against 8x8 gains on no side: 24 depth
+    // numbers, 200x200 13.2 and 12.0, 600x400 42.6 and 42.7.
+    static const int cand[][2] = {{16, 8}, {16, 6}, {8, 8}, {16, 4}, {32, 4}, {8, 7}, {8, 6},
+                                  {8, 5},  {8, 4},  {32, 2}, {16, 2}, {4, 8}, {8, 3}, {8, 2},
+                                  {4, 4},  {16, 1}, {8, 1},  {4, 2},  {4, 1}};
     if (want_w || want_h) {
         if (!(want_w == 4 || want_w == 8 || want_w == 16 || want_w == 32) || want_h < 1 ||
             want_h > 8)

@@ -57,3 +57,39 @@ def test_tile_edges_exact(D, tile, bt):
         X, flow, status = gc.solve_costs(torch.from_numpy(C).cuda(), p, o)
         assert int(status.item()) == gc.GS_OK and int(flow.item()) == ref["flow"]
         assert np.array_equal(X.cpu().numpy(), ref["labels"])
+
+
+@pytest.mark.parametrize("bt,D,shape", [
+    (512, 17, (16, 8)), (512, 18, (16, 6)), (512, 21, (16, 6)), (512, 22, (8, 8)),
+    (512, 33, (8, 8)), (512, 34, (8, 7)),
+    (512, 37, (8, 7)), (512, 38, (8, 6)), (512, 41, (8, 6)), (512, 42, (8, 5)),
+    (512, 49, (8, 5)), (512, 50, (8, 4)), (512, 65, (8, 4)), (512, 66, (8, 3)),
+    (256, 9, (16, 8)), (256, 10, (8, 8)), (256, 17, (8, 8)),
+    (256, 18, (8, 6)), (256, 22, (8, 5)),
+])
+def test_own_shape_fills_the_threads(bt, D, shape):
+    """The library's own tile at both ends of each range of blocks of four
+    layers: at most one block per thread."""
+    from paper_1803_01516_gb300 import build
+    build.build()
+    from paper_1803_01516_gb300 import gazecut as gc
+    p = gc.Params(w=2 * (D - 1) + 64, h=40, D=D, tau=30, lam=3)
+    info = gc.gs_tile_info(p, gc.SolveOpts(cta_threads=bt))
+    assert (info["tile_w"], info["tile_h"]) == shape
+    assert info["tile_w"] * info["tile_h"] * ((D + 2) // 4) <= bt
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D,bt", [(10, 256), (18, 512), (22, 512), (25, 256), (34, 512), (38, 512),
+                                  (45, 512), (66, 512)])
+def test_own_shape_exact(D, bt):
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1803_01516_gb300 import gazecut as gc
+    h, ng = 23, 35                                   # no tile divides either
+    C = np.random.default_rng(D).integers(0, 31, size=(h, ng, D)).astype(np.int32)
+    p = gc.Params(w=ng + 2 * (D - 1), h=h, D=D, tau=0, lam=4, inhibit=37)
+    ref = oracle.solve(C, 4, 37, 1)
+    X, flow, status = gc.solve_costs(torch.from_numpy(C).cuda(), p, gc.SolveOpts(cta_threads=bt))
+    assert int(status.item()) == gc.GS_OK and int(flow.item()) == ref["flow"]
+    assert np.array_equal(X.cpu().numpy(), ref["labels"])
