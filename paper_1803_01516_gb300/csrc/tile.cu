@@ -1726,6 +1726,22 @@ __device__ __forceinline__ void visit_tile(const SolveArgs &a, PairCtl *c, const
     }
 }
 
+// What bounds a launch: the chain of dependent instructions of its tile visits
+// (a fifth to a quarter of the issue slots are used, DRAM at a few percent) and,
+// where a step has few items, the wait for its last one (62 % of the block time
+// at 384x288x16, 10 % at 640x480x64) with a hand-over of about 4 us.  Visits in
+// us as staging + work + write-back, measured in a copy with counters, with a
+// node per lane and a warp's own lists -> as it is:
+//   384x288x16 (8x8 tiles, 2 x 256 threads an SM): sweep 2.7 + 11.7 + 2.8 -> 2.5 +
+//     9.1 + 2.5, relabel 1.3 + 4.3 + 1.7 -> 1.0 + 3.1 + 1.0, first pass 5.8 + 5.2 + 0.5
+//     -> 2.7 + 4.6 + 0.4; the solve 13.1 -> 10.6 ms
+//   640x480x64 (8x4, 512 threads): sweep 4.7 + 8.7 + 2.6 -> 3.9 + 9.8 + 2.7 for a third
+//     fewer visits, relabel 2.1 + 16.0 + 1.9 -> 1.6 + 4.9 + 1.1, first pass 8.2 + 5.8 +
+//     0.4 -> 4.4 + 4.5 + 0.3; the solve 225 -> 106 ms
+// An iteration takes 0.72 us for up to 64 nodes in 512 threads (0.66 by one warp):
+// loads 97 cycles, admissibility and scan 230, pushes 290, the place in the next
+// list 230, barrier and loop 200.
+//
 // TPT: blocks of own nodes per thread, the most any pair of the launch needs.
 // Blocks of 256 or 512 threads; 128 registers a thread leave room for two or
 // one of them per SM.
