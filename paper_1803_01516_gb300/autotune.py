@@ -164,11 +164,17 @@ def _defaults() -> dict:
 
 def tuned_opts(p: gc.Params, tune_if_missing: bool = False, **kw) -> gc.SolveOpts:
     """Solve options for p from the cache (library defaults when absent)."""
-    entry = _load().get(bucket(p)) or _defaults().get(bucket(p))
+    entry = _load().get(bucket(p))
+    shipped = entry is None
+    if shipped:
+        entry = _defaults().get(bucket(p))
     if entry is None and tune_if_missing:
-        entry = tune(p)
+        entry, shipped = tune(p), False
     if entry is None:
-        entry = _nearest(_load(), p) or _nearest(_defaults(), p)
+        entry = _nearest(_load(), p)
+        shipped = entry is None
+        if shipped:
+            entry = _nearest(_defaults(), p)
     if entry is None:
         return gc.SolveOpts(**kw)
     best = entry["best"]
@@ -176,6 +182,11 @@ def tuned_opts(p: gc.Params, tune_if_missing: bool = False, **kw) -> gc.SolveOpt
     tw, th = (best[3], best[4]) if len(best) >= 5 else (0, 0)
     ti = best[5] if len(best) >= 6 else 0          # tail iterations (0: library default)
     bt = best[6] if len(best) >= 7 else 0          # threads per block (0: library default)
+    if shipped and tw * th * ((p.D + 2) // 4) > (bt or 512):
+        # a bucket spans several chain lengths; where its shape has more blocks
+        # of four layers than threads the library's own shape is the faster one
+        # (18 to 20 depth numbers, 256 threads: 800x500 91 ms at 8x8, 68 at 8x6)
+        tw = th = 0
     o = gc.SolveOpts(sweeps_per_relabel=spr, local_iters=li, relabel_passes=rp, tile_w=tw,
                      tile_h=th, tail_iters=ti, cta_threads=bt, **kw)
     try:

@@ -93,3 +93,25 @@ def test_own_shape_exact(D, bt):
     X, flow, status = gc.solve_costs(torch.from_numpy(C).cuda(), p, gc.SolveOpts(cta_threads=bt))
     assert int(status.item()) == gc.GS_OK and int(flow.item()) == ref["flow"]
     assert np.array_equal(X.cpu().numpy(), ref["labels"])
+
+
+@pytest.mark.parametrize("w,h,D,shape", [(384, 288, 16, (8, 8)), (400, 300, 17, (8, 8)),
+                                         (400, 300, 18, (8, 6)), (400, 300, 20, (8, 6)),
+                                         (500, 400, 8, (16, 8)), (500, 400, 9, (16, 8))])
+def test_shipped_shape_fills_the_threads(w, h, D, shape, monkeypatch, tmp_path):
+    """Shipped entries at both ends of their bucket's chain lengths: at most one
+    block of layers per thread; a shape from the caller's own cache stays."""
+    import json
+    from paper_1803_01516_gb300 import build
+    build.build()
+    from paper_1803_01516_gb300 import autotune
+    from paper_1803_01516_gb300 import gazecut as gc
+    monkeypatch.setenv("GAZECUT_TUNE_CACHE", str(tmp_path / "cache.json"))
+    p = gc.Params(w=w, h=h, D=D, tau=30, lam=10)
+    o = autotune.tuned_opts(p)
+    info = gc.gs_tile_info(p, o)
+    assert o.cta_threads == 256 and (info["tile_w"], info["tile_h"]) == shape
+    with open(autotune.cache_path(), "w") as f:
+        json.dump({autotune.bucket(p): {"best": [16, 8, 0, 8, 8, 16, 256]}}, f)
+    o = autotune.tuned_opts(p)
+    assert (o.tile_w, o.tile_h) == (8, 8)
