@@ -25,11 +25,17 @@ import torch
 from . import gazecut as gc
 from . import synth
 
-SCHEDULES = [(spr, li, rp, tf) for spr in (8, 16, 32, 64) for li in (4, 8, 16) for rp in (4, 8, 16)
-             for tf in (2, 4)]       # tf: tail iterations = tf x local iterations
-SHAPES = [(16, 8), (16, 6), (8, 8), (16, 4), (32, 4), (8, 7), (8, 6), (8, 5), (8, 4), (16, 2),
+# Relabel passes 0 is the library's rule (1024 / sites of a tile); the fixed
+# caps bracket it.  tf: tail iterations = tf x local iterations.
+SCHEDULES = [(spr, li, rp, tf) for spr in (8, 16, 32, 64) for li in (4, 8, 16)
+             for rp in (0, 8, 16, 32) for tf in (2, 4)]
+# 0 x 0 is the library's own shape
+SHAPES = [(0, 0), (16, 8), (16, 6), (8, 8), (16, 4), (32, 4), (8, 7), (8, 6), (8, 5), (8, 4), (16, 2),
           (8, 2), (4, 4)]
 CTA_THREADS = (512, 256)     # one block per SM, or two half-size blocks
+# Entries name the solver they were measured on: a schedule tuned for an earlier
+# one can be slower than the library's own.
+SOLVER = 2
 
 
 def cache_path() -> str:
@@ -64,6 +70,13 @@ def _nearest(table: dict, p: gc.Params):
 
 
 def _load() -> dict:
+    """The cache's entries: those measured on this solver, and those written by
+    hand (without measurements)."""
+    return {k: e for k, e in _load_all().items()
+            if not (isinstance(e, dict) and "all_ms" in e) or e.get("solver") == SOLVER}
+
+
+def _load_all() -> dict:
     try:
         with open(cache_path()) as f:
             return json.load(f)
@@ -112,10 +125,13 @@ def _time_config(p: gc.Params, pairs, cfg, reps: int = 2) -> float:
 
 
 def tune(p: gc.Params, n_pairs: int = 2, save: bool = True, pairs=None) -> dict:
-    """Tile shape and block size first (default schedule), then the schedule on
-    the best of those, each measured on `pairs` -- the caller's own image
-    pairs of p's size, a list of (left, right) uint8 device tensors -- or, by
-    default, on n_pairs synthetic pairs of that size.  An entry is
+    """Tile shape and block size first (the library's schedule, whose relabel cap
+    follows the tile: under one fixed cap large tiles win for the wrong
+    reason), then the schedule on the best of those, each measured on `pairs`
+    -- the caller's own image pairs of p's size, a list of (left, right) uint8
+    device tensors -- or, by default, on n_pairs synthetic pairs of that size.
+    The library's defaults and the shipped entry are among the candidates, so
+    the result is never one that measured slower than either.  An entry is
     [sweeps_per_relabel, local_iters, relabel_passes, tile_w, tile_h,
     tail_iters, cta_threads]."""
     if pairs is None:
@@ -135,19 +151,23 @@ def tune(p: gc.Params, n_pairs: int = 2, save: bool = True, pairs=None) -> dict:
                 raise ValueError(f"tune: pair of shape {tuple(L.shape)} / {tuple(R.shape)}, "
                                  f"expected {(p.h, p.w)}")
     results = {}
-    for tw, th in SHAPES:
-        for bt in CTA_THREADS:
-            results[f"16,8,8,{tw},{th},0,{bt}"] = _time_config(p, pairs, (16, 8, 8, tw, th, 0, bt))
-    first = [int(x) for x in min(results, key=results.get).split(",")]
-    tw, th, bt = first[3], first[4], first[6]
+    first = [(16, 8, 0, tw, th, 0, bt) for tw, th in SHAPES for bt in CTA_THREADS]
+    o = _shipped_opts(p)
+    first.append((o.sweeps_per_relabel, o.local_iters, o.relabel_passes, o.tile_w, o.tile_h,
+                  o.tail_iters, o.cta_threads))
+    for cfg in first:
+        if cfg not in results:
+            results[cfg] = _time_config(p, pairs, cfg)
+    tw, th, bt = (min(results, key=results.get)[i] for i in (3, 4, 6))
     for spr, li, rp, tf in SCHEDULES:
-        key = f"{spr},{li},{rp},{tw},{th},{tf * li},{bt}"
-        if key not in results:
-            results[key] = _time_config(p, pairs, (spr, li, rp, tw, th, tf * li, bt))
+        cfg = (spr, li, rp, tw, th, tf * li, bt)
+        if cfg not in results:
+            results[cfg] = _time_config(p, pairs, cfg)
     best = min(results, key=results.get)
-    entry = {"best": [int(x) for x in best.split(",")], "ms": results[best], "all_ms": results}
+    entry = {"best": list(best), "ms": results[best], "solver": SOLVER,
+             "all_ms": {",".join(map(str, c)): ms for c, ms in results.items()}}
     if save:
-        d = _load()
+        d = _load_all()
         d[bucket(p)] = entry
         _save(d)
     return entry
@@ -165,28 +185,34 @@ def _defaults() -> dict:
 def tuned_opts(p: gc.Params, tune_if_missing: bool = False, **kw) -> gc.SolveOpts:
     """Solve options for p from the cache (library defaults when absent)."""
     entry = _load().get(bucket(p))
-    shipped = entry is None
-    if shipped:
-        entry = _defaults().get(bucket(p))
-    if entry is None and tune_if_missing:
-        entry, shipped = tune(p), False
-    if entry is None:
+    if entry is None and tune_if_missing and bucket(p) not in _defaults():
+        entry = tune(p)
+    if entry is None and bucket(p) not in _defaults():
         entry = _nearest(_load(), p)
-        shipped = entry is None
-        if shipped:
-            entry = _nearest(_defaults(), p)
+    return _shipped_opts(p, **kw) if entry is None else _entry_opts(p, entry, **kw)
+
+
+def _shipped_opts(p: gc.Params, **kw) -> gc.SolveOpts:
+    """Solve options for p from the shipped table alone."""
+    entry = _defaults().get(bucket(p)) or _nearest(_defaults(), p)
     if entry is None:
         return gc.SolveOpts(**kw)
+    best = list(entry["best"])
+    bt = best[6] if len(best) >= 7 else 0
+    if len(best) >= 5 and best[3] * best[4] * ((p.D + 2) // 4) > (bt or 512):
+        # a bucket spans several chain lengths; where its shape has more blocks
+        # of four layers than threads the library's own shape is the faster one
+        # (18 to 20 depth numbers, 256 threads: 800x500 91 ms at 8x8, 68 at 8x6)
+        best[3] = best[4] = 0
+    return _entry_opts(p, {"best": best}, **kw)
+
+
+def _entry_opts(p: gc.Params, entry: dict, **kw) -> gc.SolveOpts:
     best = entry["best"]
     spr, li, rp = best[:3]
     tw, th = (best[3], best[4]) if len(best) >= 5 else (0, 0)
     ti = best[5] if len(best) >= 6 else 0          # tail iterations (0: library default)
     bt = best[6] if len(best) >= 7 else 0          # threads per block (0: library default)
-    if shipped and tw * th * ((p.D + 2) // 4) > (bt or 512):
-        # a bucket spans several chain lengths; where its shape has more blocks
-        # of four layers than threads the library's own shape is the faster one
-        # (18 to 20 depth numbers, 256 threads: 800x500 91 ms at 8x8, 68 at 8x6)
-        tw = th = 0
     o = gc.SolveOpts(sweeps_per_relabel=spr, local_iters=li, relabel_passes=rp, tile_w=tw,
                      tile_h=th, tail_iters=ti, cta_threads=bt, **kw)
     try:
