@@ -4,9 +4,11 @@
 
 namespace gs {
 
+constexpr int kSumWords = 32;       // words of static shared memory of block_sum_u64, a warp one
+
 __device__ __forceinline__ void block_sum_u64(unsigned long long v, unsigned long long *out) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    __shared__ unsigned long long red[32];
+    __shared__ unsigned long long red[kSumWords];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();
     if (lane == 0) red[wid] = v;
@@ -394,12 +396,14 @@ int gs_build_graph_flags(const int32_t *cost, const gs_params *p, int32_t flags,
     k_header<<<1, 1, 0, st>>>(s.hdr, g, p->inhibit, p->vertical_inhibit);
     k_dir_sums<<<grid_for((int64_t)g.ng * g.h), 256, 0, st>>>(cost, g, s.hdr);
     k_decide<<<1, 1, 0, st>>>(s.hdr, p->direction);
-    // chains too long for 48 KB of staged costs (more than 380 depth numbers)
-    // read them in place
+    // A launch without an opt-in has 48 KB of shared memory, the kernel's static
+    // sums included: chains too long for the rest (more than 381 depth numbers)
+    // read their costs in place.
     const size_t staged = 32 * (size_t)(g.D | 1) * sizeof(int32_t);
+    const size_t room = 48 * 1024 - kSumWords * sizeof(unsigned long long);
     const int64_t blocks = (int64_t)g.h * (g.P / 32);
     if (blocks > 0x7fffffff) return GS_ERR_INVAL;
-    if (staged <= 48 * 1024)
+    if (staged <= room)
         k_build<true><<<(int)blocks, 32 * kBuildWarps, staged, st>>>(
             cost, g, s, status, flags & GS_BUILD_CHAIN_PREFLOW);
     else
