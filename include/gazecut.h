@@ -102,7 +102,8 @@ typedef struct gs_solve_opts {
                                     (0: 1024 / sites of a tile, 8 to 64); the relabel that
                                     decides termination always runs to its fixed point */
     int32_t tail_iters;          /* TILED: local iterations per tile visit once few nodes
-                                    are active (0: 2 x local_iters) */
+                                    are active (0: 2 x local_iters, 4 x in
+                                    GS_MODE_FIXED_SWEEPS) */
     int32_t tile_w, tile_h;      /* TILED: sites per tile along W (4, 8, 16 or 32) and
                                     rows per tile (1..8); 0, 0: chosen by the library.
                                     A shape that does not fit shared memory is refused
