@@ -545,17 +545,26 @@ __device__ __forceinline__ bool relax_tile(const SolveArgs &a, int32_t *sm, cons
             stop = outer >= 2 && seen + margin >= items;
             seen = *(volatile const unsigned *)done_ctr;
         }
-        // (the counts are read before the heights they count changes of)
+        // A warp that has seen a count must see the heights it counts, or it
+        // would rest on old ones after the barrier too: the count is read before
+        // the heights, and a writer's heights are visible before it counts them,
+        // with a fence on either side (the warp barriers carry it to all lanes).
         const uint32_t now = chg[watch];
         const bool fresh = __any_sync(0xffffffffu, now != last);
         last = now;
         if (fresh || outer == 0) {
+            __threadfence_block();
+            __syncwarp();
 #pragma unroll
             for (int u = 0; u < TPT; u++) {
                 const bool ch = cell[u] > 0 && relax_block<TWC>(l, sm + cell[u], nl[u], mk[u]);
                 if (__any_sync(0xffffffffu, ch)) {
                     changed = 1;
-                    if (uniform ? lane == 0 : ch) red_add_smem((int32_t *)&chg[blk[u] + 1], 1);
+                    __syncwarp();
+                    if (uniform ? lane == 0 : ch) {
+                        __threadfence_block();
+                        red_add_smem((int32_t *)&chg[blk[u] + 1], 1);
+                    }
                 }
             }
         }
