@@ -409,8 +409,16 @@ GS_API int gs_block_descent(const int32_t *cost, const gs_params *p, int32_t b,
 
 /* Tile shape the TILED engine uses for these params and options: host
  * int32[4] = {sites per tile along W, rows per tile, number of tiles, bytes of
- * the tile's nine fields in shared memory}.  GS_ERR_INVAL if the requested shape does not fit. */
+ * the nine fields of the tile's nodes and halo}.  The fields are what the shape
+ * rules go by (at most 180 KB); gs_tile_smem_bytes is what a launch takes.
+ * GS_ERR_INVAL if the requested shape does not fit. */
 GS_API int gs_tile_info(const gs_params *p, const gs_solve_opts *o, int32_t *out);
+
+/* Dynamic shared memory of a block of the TILED engine's launch for these params
+ * and options, bytes: the tile's fields, the padding between its rows and its
+ * lists.  Another 1 KB at most is static.  0 if the params are invalid or the
+ * requested shape does not fit. */
+GS_API size_t gs_tile_smem_bytes(const gs_params *p, const gs_solve_opts *o);
 
 /* Number of kernels this library has launched in this process so far. */
 GS_API int64_t gs_kernel_launches(void);

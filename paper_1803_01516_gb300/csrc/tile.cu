@@ -1876,10 +1876,12 @@ static size_t field_bytes(const Geom &g, int TW, int TH, int bt) {
 // Tile shape: whole chains (all K layers), TW sites x TH rows, the nine fields
 // within 180 KB; one block of kBlk layers per thread, or two.  The library's
 // own choice prefers one, and with 256-thread blocks fields within 80 KB, so
-// that two tiles fit an SM (long chains fall back to one).  A tile takes up to
-// 15 % more shared memory than its fields (the padding between rows, the lists
-// of active nodes), which stays within a block's 227 KB.  `fields` returns
-// field_bytes of the shape, `smem` what the kernel needs.
+// that two tiles fit an SM (long chains fall back to one).  The kernel takes more
+// shared memory than the fields (a layer of padding between rows of sites, the
+// lists of active nodes): 216124 bytes for 184320 at the most, a third more at
+// 9 depth numbers, 3.4 times as much at 2, where the padding is as large as the
+// chains.  `fields` returns field_bytes of the shape, `smem` what the kernel
+// needs, within a block's 227 KB.
 static bool pick_tile(const Geom &g, TileGeom &t, int &tpt, size_t &smem, int want_w = 0,
                       int want_h = 0, int bt = kTileThreads, size_t *fields = nullptr) {
     const size_t budgets[2] = {(bt == 256 && !want_w ? 80 : 180) * size_t(1024), 180 * 1024};
@@ -2121,6 +2123,17 @@ extern "C" int gs_tile_info(const gs_params *p, const gs_solve_opts *o, int32_t 
     out[2] = t.T;
     out[3] = (int32_t)fields;
     return GS_OK;
+}
+
+extern "C" size_t gs_tile_smem_bytes(const gs_params *p, const gs_solve_opts *o) {
+    gs::Geom g;
+    gs::TileGeom t;
+    int tpt;
+    size_t smem;
+    if (!o || gs::make_geom(p, &g) != GS_OK ||
+        !gs::pick_tile(g, t, tpt, smem, o->tile_w, o->tile_h, gs::cta_threads(g, o)))
+        return 0;
+    return smem;
 }
 
 // ------------------------------------------------------------ batched ABI ---

@@ -34,7 +34,7 @@ EXPORTS = [
     "gs_cost_add_at_labels", "gs_batch_workspace_bytes", "gs_solve_batched",
     "gs_delegate_params", "gs_delegate_cost", "gs_skin_bounds", "gs_build_graph_skin",
     "gs_build_graph_flags", "gs_check_solve_opts", "gs_stereo_cost_volume_rgb",
-    "gs_level2_start", "gs_block_descent",
+    "gs_level2_start", "gs_block_descent", "gs_tile_smem_bytes",
 ]
 GS_BUILD_CHAIN_PREFLOW = 1
 
@@ -140,6 +140,7 @@ def lib():
             "gs_kernel_launches": ([], I64),
             "gs_noalloc_scratch_bytes": ([], SZ),
             "gs_tile_info": ([pp, po, P], ctypes.c_int),
+            "gs_tile_smem_bytes": ([pp, po], SZ),
             "gs_stereo_cost_volume_f32": ([P, P, I32, pp, F, F, F, F, P, P], ctypes.c_int),
             "gs_energy_backward": ([P, pp, F, P, P, P], ctypes.c_int),
             "gs_cost_volume_f32_backward": ([P, P, I32, pp, F, F, F, P, P, P], ctypes.c_int),
@@ -334,10 +335,20 @@ def gs_kernel_launches() -> int:
 
 
 def gs_tile_info(p: Params, o: SolveOpts | None = None) -> dict:
+    """Tile shape of the persistent solver.  ``smem_bytes`` are the tile's nine
+    fields, the size its shape rules go by; ``launch_smem_bytes`` is what a
+    block of the launch takes."""
     out = (ctypes.c_int32 * 4)()
     o = o or SolveOpts()
     _check(lib().gs_tile_info(ctypes.byref(p.c()), ctypes.byref(o.c()), out), "gs_tile_info")
-    return {"tile_w": out[0], "tile_h": out[1], "tiles": out[2], "smem_bytes": out[3]}
+    return {"tile_w": out[0], "tile_h": out[1], "tiles": out[2], "smem_bytes": out[3],
+            "launch_smem_bytes": gs_tile_smem_bytes(p, o)}
+
+
+def gs_tile_smem_bytes(p: Params, o: SolveOpts | None = None) -> int:
+    """Dynamic shared memory of a block of the persistent launch (0: no tile fits)."""
+    o = o or SolveOpts()
+    return int(lib().gs_tile_smem_bytes(ctypes.byref(p.c()), ctypes.byref(o.c())))
 
 
 def gs_noalloc_scratch_bytes() -> int:
