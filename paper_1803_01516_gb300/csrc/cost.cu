@@ -311,12 +311,13 @@ __device__ __forceinline__ int pixel_dx(const uint8_t *row, int x, int w) {
 }
 
 // One block per (row y, tile of kCostTW sites).  The two image segments are
-// staged once (unless the depth range is too long for it) as (pixel, pixel difference I[x+1] - I[x-1]) pairs in one word,
-// so a cross point takes two shared loads; the output block [TW][D] is
-// contiguous and is written VEC entries a thread (int4 where the block starts
-// on a 16-byte boundary and holds whole quadruples).  Bound by the output:
-// 1154x720 sites x 64 depth numbers, 213 MB, took 185 us when every cross point
-// read its eight image bytes from global memory, and takes 60 us this way.
+// staged once (unless the depth range is too long for it) as (pixel, pixel
+// difference I[x+1] - I[x-1]) pairs in one word, so a cross point takes two
+// shared loads; the output block [TW][D] is contiguous and is written VEC entries
+// a thread (int4 where the block starts on a 16-byte boundary and holds whole
+// quadruples).  Bound by the output: 1154x720 sites x 64 depth numbers, 213 MB,
+// took 185 us when every cross point read its eight image bytes from global
+// memory, and takes 60 us this way.
 template <int VEC, bool STAGED>
 __global__ void k_cost_volume_f32(const uint8_t *__restrict__ L, const uint8_t *__restrict__ R,
                                   int pitch, int w, int ng, int D, int dis0, float w1, float w2,

@@ -13,12 +13,12 @@
 // of lambda |d| on |d| <= 1 (infinite beyond) with (lambda + inhibit) |d|, so a
 // line of n labels takes a three-point minimum and one running minimum each
 // way.  Moving from row to row costs 2 bw n^bw steps, instead of n^(2 bw) for
-// all pairs of states or bw n^(bw+1) for all pairs of labels.  Forward and backward passes give every row state's
-// min-marginal; the smallest label a site takes in any minimiser, read from
-// the states whose min-marginal equals the minimum, is the site's label in the
-// component-wise smallest minimiser (the minimisers of this convex-prior
-// energy form a lattice under component-wise min), the same canonical answer
-// as the minimal source set of the block's cut.
+// all pairs of states or bw n^(bw+1) for all pairs of labels.  Forward and
+// backward passes give every row state's min-marginal; the smallest label a site
+// takes in any minimiser, read from the states whose min-marginal equals the
+// minimum, is the site's label in the component-wise smallest minimiser (the
+// minimisers of this convex-prior energy form a lattice under component-wise
+// min), the same canonical answer as the minimal source set of the block's cut.
 #include "gs_internal.cuh"
 
 namespace gs {

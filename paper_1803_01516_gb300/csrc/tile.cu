@@ -1747,9 +1747,15 @@ __device__ __forceinline__ void visit_tile(const SolveArgs &a, PairCtl *c, const
 //   640x480x64 (8x4, 512 threads): sweep 4.7 + 8.7 + 2.6 -> 3.9 + 9.8 + 2.7 for a third
 //     fewer visits, relabel 2.1 + 16.0 + 1.9 -> 1.6 + 4.9 + 1.1, first pass 8.2 + 5.8 +
 //     0.4 -> 4.4 + 4.5 + 0.3; the solve 225 -> 106 ms
-// An iteration takes 0.72 us for up to 64 nodes in 512 threads (0.66 by one warp):
-// loads 97 cycles, admissibility and scan 230, pushes 290, the place in the next
-// list 230, barrier and loop 200.
+// An iteration takes 0.72 us for up to 64 nodes in 512 threads (0.66 by one warp).
+// A warp's discharge is 0.45 us of it: loads 97 cycles, admissibility and scan 230,
+// pushes 290, the place in the next list 230, the entries' stores 82.  The other
+// 0.27 us are the loop, the list's length and the barrier with the wait for the
+// slowest warp.
+// Registers: one block of nodes per thread takes all 128 and spills 32 bytes; two
+// (explicit shapes only, and every pair of a batch that holds one) spill 884, and
+// still take half the time of the node-per-lane code on the same shapes
+// (500x400x48, 8x8: 43 against 84 ms).
 //
 // TPT: blocks of own nodes per thread, the most any pair of the launch needs.
 // Blocks of 256 or 512 threads; 128 registers a thread leave room for two or
